@@ -5,32 +5,48 @@
 // 128-token query tile of two q-heads of the same kv-head (one head when the
 // group size is 1) over a range of 128-key KV tiles; both Q tiles share every
 // K/V tile the CTA loads.  Per Q tile t the work is a chain
-// S_t = Q_t K^T -> softmax -> P_t (bf16, written over S_t in TMEM) ->
-// O_t += P_t V, and the two tiles' chains interleave on the tensor core.
+// S_t = Q_t K^T -> softmax -> P_t (bf16, in TMEM) -> O_t += P_t V, and the
+// two tiles' chains interleave on the tensor core.
 // TMEM, the barriers and the K/V rings live across items, so an item's
 // epilogue overlaps the next item's first Q K^T and its K/V loads.
+// TMEM (512 columns) holds one S of 128 columns, which the two tiles use in
+// turn, and apart from it P_0, P_1 (64 each) and O_0, O_1 (128 each).  A
+// softmax thread takes its whole S row into registers first, so S is free
+// for the other tile's Q K^T ~200 cycles after it is complete, long before
+// P of the row exists; with P over S's own columns (two S buffers of 128,
+// no room apart) Q K^T had to wait for the P V that reads P, and the chain
+// softmax -> P V -> Q K^T set the pace: 4340 cycles a KV tile of both Q
+// tiles (2048 of them MMA), the two softmax warpgroups held apart by a turn
+// barrier.  Now they overlap, 3100-3300 cycles a KV tile, and what is left
+// is the loop Q K^T (540 in issue) -> S seen (250) -> S read out (200) ->
+// next Q K^T (165-300) twice a tile, with P V in its gaps.
 // Warp roles (512 threads, four warpgroups):
 //   warps 0-3   TMA producers: warps 0/1 fetch pages 0-3 / 4-7 of each K
 //               tile (3-stage ring), warps 2/3 those of each V tile (2
 //               stages), through the block table.  One issuing thread moves
 //               only ~7 B/clk of small TMA boxes on GB300, so every tile is
 //               fetched by two threads.
-//   warps 4, 5  MMA issuers, one thread per Q tile: S_t = Q_t K^T (A = Q in
-//               shared memory) and O_t += P_t V (A = P in TMEM); Q K^T for the
-//               next tile is issued once P V has consumed P.
+//   warp 4      Q K^T issuer (one thread): S = Q_t K^T (A = Q in shared
+//               memory) for t = 0, 1, as soon as S has been read out.
+//   warp 5      P V issuer (one thread): O_t += P_t V (A = P in TMEM).  A
+//               batch goes out behind the Q K^T batch after the next one
+//               (see there).  One thread for both took 4400 cycles a KV
+//               tile: a thread that issues MMAs is held up until the tensor
+//               core has taken them, so its waits and commits are gaps.
 //   warp 6      Q loader: Q_t of the next item once the last Q K^T of the
 //               current item on tile t has completed.
 //   warps 8-11  softmax for tile 0, warps 12-15 for tile 1: each thread owns
 //               one query row (its TMEM lane), loads its S row, masks by
 //               absolute position, runs the online softmax in fp32 (exp2
 //               domain) and stores P back to TMEM; at the end of an item it
-//               writes O (or a piece's partial).  The two warpgroups take
-//               turns, tile 0 then tile 1, so that one tile's softmax runs
-//               under the other tile's MMAs.
+//               writes O (or a piece's partial).
 // Registers move from the producer/MMA warpgroups to the softmax warpgroups
 // with setmaxnreg.  The running max is only raised (and O rescaled in TMEM)
 // when it grows by more than 2^8; until then the stale max keeps every
 // exponent <= 2^8, and the final O / l is exact either way.
+// (16384 tokens over an empty prefix, 16/2 heads: 922 us before, 735 now;
+// 8616 over 16384: 1221 -> 985; the ratio shrinks by a few percent in a long
+// run, where the faster kernel draws the clock down.)
 // The host plan may cut a long (query tile, head slot) unit into pieces on
 // consecutive CTAs (stream-K): each piece writes its partial (m, l, O) to the
 // workspace, and prefill_merge_kernel, launched after this kernel, combines
@@ -70,10 +86,11 @@ enum : int {
     B_VFULL = B_KEMPTY + kNK,
     B_VEMPTY = B_VFULL + kNV,
     B_SFULL = B_VEMPTY + kNV,  // [tile]
-    B_PFULL = B_SFULL + 2,     // [tile]
+    B_SFREE = B_SFULL + 2,     // the S columns have been read out
+    B_PFULL = B_SFREE + 1,     // [tile]
     B_ODONE = B_PFULL + 2,     // [tile]
-    B_TURN = B_ODONE + 2,      // [tile]: the softmax warpgroups take turns
-    B_DRAIN = B_TURN + 2,
+    B_QKI = B_ODONE + 2,       // [4]: Q K^T batch n, issued (n mod 4)
+    B_DRAIN = B_QKI + 4,
     B_COUNT = B_DRAIN + 1
 };
 constexpr uint32_t kOffTmem = kOffBar + B_COUNT * 8;
@@ -81,7 +98,10 @@ constexpr uint32_t kOffAbort = kOffTmem + 4;
 static_assert(kOffAbort + 4 <= kOffBar + 256, "barrier area");
 constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024;  // + alignment slack
 static_assert(kSmemBytes <= 232448, "shared memory per CTA");
-constexpr uint32_t kTmemCols = 512;  // tile t: S/P at t*256, O at t*256 + 128
+constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kColS = 0;    // one S (128 columns) that the two tiles use in turn
+constexpr uint32_t kColP = 128;  // P of tile t at kColP + 64 t
+constexpr uint32_t kColO = 256;  // O of tile t at kColO + 128 t
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
 constexpr int kThreads = 512;
 constexpr int kMmaWarp = 4;       // warps 4..7 form the MMA warpgroup
@@ -113,30 +133,42 @@ __device__ __forceinline__ void tmem_ld32_sync(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 64 TMEM columns of this warp's lanes (one S row per thread), waiting for
-// completion before the registers are used.
-__device__ __forceinline__ void tmem_ld64_sync(uint32_t taddr, float (&v)[64]) {
-    uint32_t r[64];
+// 32 TMEM columns of this warp's lanes (one row per thread), issued only: the
+// values exist after tmem_wait_ld() and tmem_use32()
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, float *r) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x64.b32 "
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,"
-        "%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,"
-        "%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-          "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-          "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-          "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]),
-          "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]),
-          "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]),
-          "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]),
-          "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
+          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]),
+          "=f"(r[15]), "=f"(r[16]), "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]),
+          "=f"(r[22]), "=f"(r[23]), "=f"(r[24]), "=f"(r[25]), "=f"(r[26]), "=f"(r[27]), "=f"(r[28]),
+          "=f"(r[29]), "=f"(r[30]), "=f"(r[31])
         : "r"(taddr)
         : "memory");
+}
+// orders every use of the 32 values after the wait before it (the registers
+// pass through an empty statement, so no use of them can move above it)
+__device__ __forceinline__ void tmem_use32(float *r) {
 #pragma unroll
-    for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 32; i += 16)
+        asm volatile(""
+                     : "+f"(r[i]), "+f"(r[i + 1]), "+f"(r[i + 2]), "+f"(r[i + 3]), "+f"(r[i + 4]), "+f"(r[i + 5]),
+                       "+f"(r[i + 6]), "+f"(r[i + 7]), "+f"(r[i + 8]), "+f"(r[i + 9]), "+f"(r[i + 10]),
+                       "+f"(r[i + 11]), "+f"(r[i + 12]), "+f"(r[i + 13]), "+f"(r[i + 14]), "+f"(r[i + 15])
+                     :
+                     : "memory");
+}
+
+// 16 TMEM columns of this warp's lanes
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t *r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
 }
 
 __device__ __forceinline__ void tmem_st32_f(uint32_t taddr, const float (&v)[32]) {
@@ -188,6 +220,12 @@ __device__ __forceinline__ void store_row32(const P &p, int64_t orow, int c4, co
                                 pack_bf16x2(v[8 * i + 4] * inv_l, v[8 * i + 5] * inv_l),
                                 pack_bf16x2(v[8 * i + 6] * inv_l, v[8 * i + 7] * inv_l));
     }
+}
+
+// mbar_wait() by a whole warp: one vote when the phase is complete already
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int32_t *err) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
 }
 
 // The parts of a work item each role needs (read from the kernel parameters).
@@ -246,19 +284,20 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
         }
         for (int s = 0; s < kNK; ++s) {
             mbar_init(bar(B_KFULL + s), 2);      // two producer threads per tile
-            mbar_init(bar(B_KEMPTY + s), hpc);   // one release per tile's MMA thread
+            mbar_init(bar(B_KEMPTY + s), 1);
         }
         for (int s = 0; s < kNV; ++s) {
             mbar_init(bar(B_VFULL + s), 2);
-            mbar_init(bar(B_VEMPTY + s), hpc);
+            mbar_init(bar(B_VEMPTY + s), 1);
         }
         for (int t = 0; t < 2; ++t) {
             mbar_init(bar(B_SFULL + t), 1);
             mbar_init(bar(B_PFULL + t), 4);
             mbar_init(bar(B_ODONE + t), 1);
-            mbar_init(bar(B_TURN + t), 4);
         }
-        mbar_init(bar(B_DRAIN), hpc);
+        mbar_init(bar(B_SFREE), 4);
+        for (int i = 0; i < 4; ++i) mbar_init(bar(B_QKI + i), 1);
+        mbar_init(bar(B_DRAIN), 2);
         *abort_flag = 0;
         fence_mbar_init();
         prefetch_tmap(&tm_q);
@@ -339,63 +378,91 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
         }
     } else if (warp < kSoftmaxWarp0) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsSmall));
-        const int t = warp - kMmaWarp;
-        if (t < hpc && lane == 0 && w_beg < w_end) {
-            // -------------------------------------------------------- MMA issuer of Q tile t
+        if (warp == kMmaWarp && lane == 0 && w_beg < w_end) {
+            // -------------------------------------------------------- Q K^T issuer
             // descriptors are built once; advancing one operand by b bytes
             // adds b >> 4 to the start-address field (no carry: < 256 KB)
-            const uint64_t dq = smem_desc_sw128(sb + kOffQ + t * kTileBytes, 16, 1024);
+            const uint64_t dq0 = smem_desc_sw128(sb + kOffQ, 16, 1024);
             const uint64_t dk0 = smem_desc_sw128(sb + kOffK, 16, 1024);
-            const uint64_t dv0 = smem_desc_sw128(sb + kOffV, kHalf, 1024);
-            const uint32_t d_s = tmem + t * 256, d_o = tmem + t * 256 + 128;
             bool ok = true;
             int g = 0;  // KV tiles of this CTA so far
+            int n = 0;  // S tiles so far (hpc per KV tile)
             for (int w = w_beg, i = 0; ok && w < w_end; ++w, ++i) {
                 const ItemView v = item_view(p, w);
-                if (!mbar_wait(bar(B_Q + t), i & 1, p.err)) {
-                    ok = false;
-                    break;
-                }
-                for (int jj = 0; jj < v.n_kt; ++jj, ++g) {
-                    const int j = v.kt0 + jj;
-                    // ---- S_t = Q_t K(j)^T, once P V (g-1) has read P out of S's columns
+                for (int jj = 0; ok && jj < v.n_kt; ++jj, ++g) {
                     const int sk = g % kNK;
                     if (!mbar_wait(bar(B_KFULL + sk), (g / kNK) & 1, p.err)) { ok = false; break; }
-                    if (g >= 1 && !mbar_wait(bar(B_ODONE + t), (g - 1) & 1, p.err)) { ok = false; break; }
-                    tc_fence_after();
                     const uint64_t dk = dk0 + ((sk * kTileBytes) >> 4);
+                    for (int t = 0; t < hpc; ++t, ++n) {
+                        if (jj == 0 && !mbar_wait(bar(B_Q + t), i & 1, p.err)) { ok = false; break; }
+                        // the S columns, once the softmax before has read them out
+                        if (n >= 1 && !mbar_wait(bar(B_SFREE), (n - 1) & 1, p.err)) { ok = false; break; }
+                        tc_fence_after();
+                        const uint64_t dq = dq0 + ((t * kTileBytes) >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        const uint32_t o = (kk >> 2) * kHalf + (kk & 3) * 32;
-                        umma_bf16(d_s, dq + (o >> 4), dk + (o >> 4), kIdescQK, kk > 0 ? 1u : 0u);
+                        for (int kk = 0; kk < 8; ++kk) {
+                            const uint32_t o = (kk >> 2) * kHalf + (kk & 3) * 32;
+                            umma_bf16(tmem + kColS, dq + (o >> 4), dk + (o >> 4), kIdescQK, kk > 0 ? 1u : 0u);
+                        }
+                        umma_commit(bar(B_SFULL + t));
+                        mbar_arrive(bar(B_QKI + (n & 3)));  // P V (n - hpc) may follow
+                        if (t == hpc - 1) umma_commit(bar(B_KEMPTY + sk));
+                        // the item's last Q K^T frees Q_t for the next item
+                        if (jj == v.n_kt - 1) umma_commit(bar(B_QEMPTY + t));
                     }
-                    umma_commit(bar(B_SFULL + t));
-                    umma_commit(bar(B_KEMPTY + sk));
-                    // the item's last Q K^T frees Q_t for the next item
-                    if (jj == v.n_kt - 1) umma_commit(bar(B_QEMPTY + t));
-                    // ---- O_t += P_t V(j), P_t from TMEM; the item's first tile overwrites O_t
-                    const int sv = g % kNV;
-                    if (!mbar_wait(bar(B_VFULL + sv), (g / kNV) & 1, p.err)) { ok = false; break; }
-                    if (!mbar_wait(bar(B_PFULL + t), g & 1, p.err)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint64_t dv = dv0 + ((sv * kTileBytes) >> 4);
-                    const int chunks = pages_in(v.ctx_len, j);
-                    if (chunks == kPagesPerTile) {
-#pragma unroll
-                        for (int kk = 0; kk < kPagesPerTile; ++kk)
-                            umma_bf16_ts(d_o, d_s + kk * 8, dv + ((kk * 2048) >> 4), kIdescPV,
-                                         (jj > 0 || kk > 0) ? 1u : 0u);
-                    } else {
-                        for (int kk = 0; kk < chunks; ++kk)
-                            umma_bf16_ts(d_o, d_s + kk * 8, dv + ((kk * 2048) >> 4), kIdescPV,
-                                         (jj > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    umma_commit(bar(B_ODONE + t));
-                    umma_commit(bar(B_VEMPTY + sv));
                 }
             }
             if (!ok) *abort_flag = 1;
             // every MMA issued so far completes before TMEM is released
+            umma_commit(bar(B_DRAIN));
+            mbar_wait(bar(B_DRAIN), 0, p.err);
+        } else if (warp == kMmaWarp + 1 && lane == 0 && w_beg < w_end) {
+            // -------------------------------------------------------- P V issuer
+            const uint64_t dv0 = smem_desc_sw128(sb + kOffV, kHalf, 1024);
+            bool ok = true;
+            int g = 0;
+            for (int w = w_beg; ok && w < w_end; ++w) {
+                const ItemView v = item_view(p, w);
+                for (int jj = 0; ok && jj < v.n_kt; ++jj, ++g) {
+                    const int sv = g % kNV;
+                    if (!mbar_wait(bar(B_VFULL + sv), (g / kNV) & 1, p.err)) { ok = false; break; }
+                    const uint64_t dv = dv0 + ((sv * kTileBytes) >> 4);
+                    const int chunks = pages_in(v.ctx_len, v.kt0 + jj);
+                    for (int t = 0; t < hpc; ++t) {
+                        if (!mbar_wait(bar(B_PFULL + t), g & 1, p.err)) { ok = false; break; }
+                        // P V (n) goes out behind Q K^T (n + hpc): P V (n) and
+                        // the read-out of S (n + hpc - 1), which lets that
+                        // Q K^T start, are ready at about the same time, and
+                        // the tensor core would work on both batches in turn
+                        // while the softmax waits for S (809 us without this
+                        // rule, 788 with it).  Not for the last KV tile of an
+                        // item: the Q K^T after it may wait for the epilogues.
+                        // Q K^T runs at most n + 2 hpc ahead of P V (n) (the
+                        // softmax stores P (n + hpc) only after P V (n)), so
+                        // four barriers keep its phases apart.
+                        if (jj + 1 < v.n_kt) {
+                            const int gate = (g + 1) * hpc + t;
+                            if (!mbar_wait(bar(B_QKI + (gate & 3)), (gate >> 2) & 1, p.err)) { ok = false; break; }
+                        }
+                        tc_fence_after();
+                        // O_t += P_t V(j), P_t from TMEM; the item's first tile overwrites O_t
+                        const uint32_t d_p = tmem + kColP + t * 64, d_o = tmem + kColO + t * 128;
+                        if (chunks == kPagesPerTile) {
+#pragma unroll
+                            for (int kk = 0; kk < kPagesPerTile; ++kk)
+                                umma_bf16_ts(d_o, d_p + kk * 8, dv + ((kk * 2048) >> 4), kIdescPV,
+                                             (jj > 0 || kk > 0) ? 1u : 0u);
+                        } else {
+                            for (int kk = 0; kk < chunks; ++kk)
+                                umma_bf16_ts(d_o, d_p + kk * 8, dv + ((kk * 2048) >> 4), kIdescPV,
+                                             (jj > 0 || kk > 0) ? 1u : 0u);
+                        }
+                        umma_commit(bar(B_ODONE + t));
+                        if (t == hpc - 1) umma_commit(bar(B_VEMPTY + sv));
+                    }
+                }
+            }
+            if (!ok) *abort_flag = 1;
             umma_commit(bar(B_DRAIN));
             mbar_wait(bar(B_DRAIN), 0, p.err);
         } else if (warp == kQWarp && lane == 0) {
@@ -430,7 +497,7 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
         const int wq = warp & 3;
         const int r = wq * 32 + lane;  // query row == TMEM lane
         const uint32_t t_lane = tmem + (static_cast<uint32_t>(wq * 32) << 16);
-        const uint32_t t_s = t_lane + t * 256, t_o = t_lane + t * 256 + 128;
+        const uint32_t t_s = t_lane + kColS, t_p = t_lane + kColP + t * 64, t_o = t_lane + kColO + t * 128;
         const float sl2 = p.scale_log2;
         bool ok = true;
         int g = 0;  // KV tiles of this CTA so far
@@ -454,30 +521,31 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
 
             for (int jj = 0; ok && jj < n_kt; ++jj, ++g) {
                 const int j = kt0 + jj;  // absolute KV tile
-                // S_t(g) ready; it was issued after P V (g-1) completed, so O_t is stable
-                ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(bar(B_SFULL + t), g & 1, p.err));
-                // the two tiles' softmax phases alternate (tile 0 first), so one
-                // tile's softmax overlaps the other tile's MMAs instead of both
-                // competing for the exponential and FP32 pipes at once
-                if (ok && hpc == 2 && (t == 1 || g > 0))
-                    ok = __all_sync(0xffffffffu, mbar_wait(bar(B_TURN + t), (t == 0 ? g - 1 : g) & 1, p.err));
+                ok = mbar_wait_warp(bar(B_SFULL + t), g & 1, p.err);
                 if (!ok) break;
                 tc_fence_after();
                 float s[kKT];
-                {
-                    float h[64];
-                    tmem_ld64_sync(t_s, h);
 #pragma unroll
-                    for (int i = 0; i < 64; ++i) s[i] = h[i];
-                    tmem_ld64_sync(t_s + 64, h);
+                for (int q = 0; q < 4; ++q) tmem_ld32_issue(t_s + 32 * q, s + 32 * q);
+                tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 64; ++i) s[64 + i] = h[i];
-                }
+                for (int q = 0; q < 4; ++q) tmem_use32(s + 32 * q);
+                // S is in registers: the other tile's Q K^T may overwrite it
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(B_SFREE));
                 const int first_key = j * kKT;
                 if (first_key + kKT - 1 > min_pos) {
+                    // one bit per visible key: a row sees keys up to pos
+                    const int lim = pos - first_key;
 #pragma unroll
-                    for (int i = 0; i < kKT; ++i)
-                        if (first_key + i > pos) s[i] = -INFINITY;
+                    for (int q = 0; q < 4; ++q) {
+                        const int n = min(max(lim - 32 * q + 1, 0), 32);
+                        const uint32_t seen = static_cast<uint32_t>((1ull << n) - 1);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if (!((seen >> i) & 1u)) s[32 * q + i] = -INFINITY;
+                    }
                 }
                 // four independent chains over the 128 scores, two new ones per max3
                 float mx0 = fmaxf(s[0], s[4]), mx1 = fmaxf(s[1], s[5]);
@@ -500,17 +568,34 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                 const float neg_m = m_used == -INFINITY ? 0.f : -m_used;
                 const float2 sl2x2 = make_float2(sl2, sl2), negx2 = make_float2(neg_m, neg_m);
                 float2 ra = make_float2(0.f, 0.f), rb = make_float2(0.f, 0.f);
+                // P (bf16 pairs, lower key in the low half), packed as the
+                // exponentials come.  (The pass alone, two warpgroups at work:
+                // 1799 cycles with each x64 load awaited by itself and packing
+                // after the last exponential, 1392 with all loads issued
+                // together and packing in this loop.)
+                uint32_t pk[4][16];
 #pragma unroll
-                for (int i = 0; i < kKT; i += 4) {
-                    const float2 xa = fma2(make_float2(s[i], s[i + 1]), sl2x2, negx2);
-                    const float2 xb = fma2(make_float2(s[i + 2], s[i + 3]), sl2x2, negx2);
-                    s[i] = ex2(xa.x);
-                    s[i + 1] = ex2(xa.y);
-                    s[i + 2] = ex2(xb.x);
-                    s[i + 3] = ex2(xb.y);
-                    ra = add2(ra, make_float2(s[i], s[i + 1]));
-                    rb = add2(rb, make_float2(s[i + 2], s[i + 3]));
+                for (int q = 0; q < 4; ++q) {
+#pragma unroll
+                    for (int i = 0; i < 32; i += 4) {
+                        const float *v = s + 32 * q + i;
+                        const float2 xa = fma2(make_float2(v[0], v[1]), sl2x2, negx2);
+                        const float2 xb = fma2(make_float2(v[2], v[3]), sl2x2, negx2);
+                        const float2 ea = make_float2(ex2(xa.x), ex2(xa.y)), eb = make_float2(ex2(xb.x), ex2(xb.y));
+                        ra = add2(ra, ea);
+                        rb = add2(rb, eb);
+                        pk[q][i / 2] = pack_bf16x2(ea.x, ea.y);
+                        pk[q][i / 2 + 1] = pack_bf16x2(eb.x, eb.y);
+                    }
                 }
+                // P V (g-1) has read the P before and O is stable
+                if (g >= 1) {
+                    ok = mbar_wait_warp(bar(B_ODONE + t), (g - 1) & 1, p.err);
+                    if (!ok) break;
+                    tc_fence_after();
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) tmem_st16(t_p + 16 * q, pk[q]);
                 l_run = l_run * alpha + ((ra.x + ra.y) + (rb.x + rb.y));
                 if (j == last_j) {
                     // rows of the last page past the context may hold anything:
@@ -531,16 +616,8 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                         fence_proxy_async_smem();
                     }
                 }
-                // P (bf16 pairs, lower key in the low half) over the first 64 columns of S
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t pk[32];
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) pk[i] = pack_bf16x2(s[64 * h + 2 * i], s[64 * h + 2 * i + 1]);
-                    tmem_st32(t_s + 32 * h, pk);
-                }
                 if (jj >= 1 && __any_sync(0xffffffffu, need)) {
-#pragma unroll
+#pragma unroll 1
                     for (int c4 = 0; c4 < 4; ++c4) {
                         float v[32];
                         tmem_ld32_sync(t_o + c4 * 32, v);
@@ -552,10 +629,7 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(bar(B_PFULL + t));
-                    if (hpc == 2) mbar_arrive(bar(B_TURN + (t ^ 1)));  // the other tile's turn
-                }
+                if (lane == 0) mbar_arrive(bar(B_PFULL + t));
             }
 
             // ---- epilogue of the item: O_t after its last P V
@@ -569,7 +643,7 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                 if (ok) {
                     tc_fence_after();
                     const float inv_l = 1.f / l_run;
-#pragma unroll
+#pragma unroll 1
                     for (int c4 = 0; c4 < 4; ++c4) {
                         float v[32];
                         tmem_ld32_sync(t_o + c4 * 32, v);
@@ -584,7 +658,7 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                 // contiguous per chunk.
                 tc_fence_after();
                 const int64_t b = static_cast<int64_t>(wk.part) * hpc + t;
-#pragma unroll
+#pragma unroll 1
                 for (int c4 = 0; c4 < 4; ++c4) {
                     float v[32];
                     tmem_ld32_sync(t_o + c4 * 32, v);
