@@ -203,23 +203,49 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return r;
 }
 
-// 32 consecutive output columns of one row, scaled by inv_l
-template <class P>
-__device__ __forceinline__ void store_row32(const P &p, int64_t orow, int c4, const float (&v)[32], float inv_l) {
-    if (p.out_fp32) {
-        float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(p.out) + orow * kHeadDim + c4 * 32);
+// Stores 32 consecutive output columns of the warp's 32 rows, scaled by inv_l
+// (v: this thread's row; first_row: the warp's first row of the tile, whose
+// first rows_valid rows exist; dst: column 0 of the chunk in the warp's first
+// row, `stride` elements a row).  A thread holds a row, so bf16 stores of its
+// own 64 bytes would touch 32 rows an instruction; the four lanes of a quad
+// first trade 16-byte chunks (a 4 x 4 transpose by shuffles), after which an
+// instruction covers 8 rows x 64 bytes.  (One item of 16 KV tiles after the
+// other, 512 queries over 2048 keys: 25.3 us a layer with direct stores, 24.2
+// with the exchange; the same through a shared-memory buffer measured 23.8 but
+// would take a stage of the K ring.)
+__device__ __forceinline__ void store_rows(void *dst, bool fp32, int64_t stride, int lane, int first_row,
+                                           int rows_valid, const float (&v)[32], float inv_l) {
+    if (fp32) {
+        if (first_row + lane >= rows_valid) return;
+        float4 *d = reinterpret_cast<float4 *>(static_cast<float *>(dst) + lane * stride);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            dst[i] = make_float4(v[4 * i] * inv_l, v[4 * i + 1] * inv_l, v[4 * i + 2] * inv_l, v[4 * i + 3] * inv_l);
-    } else {
-        uint4 *dst = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p.out) + orow * kHeadDim + c4 * 32);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            dst[i] = make_uint4(pack_bf16x2(v[8 * i] * inv_l, v[8 * i + 1] * inv_l),
-                                pack_bf16x2(v[8 * i + 2] * inv_l, v[8 * i + 3] * inv_l),
-                                pack_bf16x2(v[8 * i + 4] * inv_l, v[8 * i + 5] * inv_l),
-                                pack_bf16x2(v[8 * i + 6] * inv_l, v[8 * i + 7] * inv_l));
+            d[i] = make_float4(v[4 * i] * inv_l, v[4 * i + 1] * inv_l, v[4 * i + 2] * inv_l, v[4 * i + 3] * inv_l);
+        return;
     }
+    uint32_t w[4][4];  // [chunk of 8 columns][pair]; afterwards [row of the quad][pair] of chunk lane & 3
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[i >> 2][i & 3] = pack_bf16x2(v[2 * i] * inv_l, v[2 * i + 1] * inv_l);
+#pragma unroll
+    for (int step = 1; step <= 2; ++step) {
+        const bool hi = (lane & step) != 0;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const int k0 = step == 1 ? 2 * x : x, k1 = k0 + step;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, hi ? w[k0][e] : w[k1][e], step);
+                w[k0][e] = hi ? got : w[k0][e];
+                w[k1][e] = hi ? w[k1][e] : got;
+            }
+        }
+    }
+    const int quad = lane & ~3;
+    __nv_bfloat16 *d = static_cast<__nv_bfloat16 *>(dst) + quad * stride + (lane & 3) * 8;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (first_row + quad + i < rows_valid)
+            *reinterpret_cast<uint4 *>(d + i * stride) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
 }
 
 // mbar_wait() by a whole warp: one vote when the phase is complete already
@@ -638,34 +664,38 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
             const PrefillSeq sq = p.seqs[wk.seq];
             const int t0 = wk.qt * kTileQ;
             const int rows_valid = min(kTileQ, sq.q_len - t0);
-            const int64_t orow = static_cast<int64_t>(sq.q_start + t0 + r) * p.n_q_heads + wk.slot * hpc + t;
             if (wk.part == kNoPart) {
                 if (ok) {
                     tc_fence_after();
                     const float inv_l = 1.f / l_run;
+                    const int64_t stride = static_cast<int64_t>(p.n_q_heads) * kHeadDim;
+                    const int64_t at = (sq.q_start + t0 + wq * 32) * stride + (wk.slot * hpc + t) * kHeadDim;
+                    uint8_t *dst = static_cast<uint8_t *>(p.out) + at * (p.out_fp32 ? 4 : 2);
+                    // (not unrolled: this code runs cold, so its length is its cost)
 #pragma unroll 1
                     for (int c4 = 0; c4 < 4; ++c4) {
                         float v[32];
                         tmem_ld32_sync(t_o + c4 * 32, v);
-                        if (r < rows_valid) store_row32(p, orow, c4, v, inv_l);
+                        store_rows(dst + c4 * (p.out_fp32 ? 128 : 64), p.out_fp32 != 0, stride, lane, wq * 32, rows_valid,
+                                   v, inv_l);
                     }
                 }
             } else if (ok) {
                 // a piece of a split unit: this range's (m, l, O) for the row;
                 // the merge kernel combines the unit's pieces after this
-                // launch.  Partial O of one (piece, head) is stored as 4 column
-                // chunks of [128 rows][32 floats], so a warp writes 4 KB
-                // contiguous per chunk.
+                // launch.  Partial O of one (piece, head) is stored as 32
+                // chunks of [128 rows][4 floats], so that a store instruction
+                // of a warp writes 512 contiguous bytes.
                 tc_fence_after();
                 const int64_t b = static_cast<int64_t>(wk.part) * hpc + t;
+                float4 *dst = reinterpret_cast<float4 *>(p.part_o) + b * (kHeadDim / 4) * kTileQ + r;
 #pragma unroll 1
                 for (int c4 = 0; c4 < 4; ++c4) {
                     float v[32];
                     tmem_ld32_sync(t_o + c4 * 32, v);
-                    float4 *dst = reinterpret_cast<float4 *>(p.part_o + ((b * 4 + c4) * kTileQ + r) * 32);
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        __stcg(dst + i, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+                        __stcg(dst + (c4 * 8 + i) * kTileQ, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
                 }
                 // two scalar stores: the paired float2 store costs the softmax loop
                 // register spills at its 200-register budget
@@ -717,8 +747,8 @@ static_assert(kDecodeThreads == 8 * 32 && kDecodeSmemBytes <= kSmemBytes,
 //   o = sum_i 2^(m_i - M) o_i / sum_i 2^(m_i - M) l_i,  M = max_i m_i
 // (m in log2 units), taking the pieces four at a time with the running
 // maximum (exact up to rounding).  One thread per (query row, 4 columns):
-// CTA (unit, head t, chunk c4, quarter) covers 32 rows x 32 columns, so a
-// warp reads 512 contiguous bytes of a partial chunk.
+// CTA (unit, head t, chunk c4, quarter) covers 32 rows x 32 columns; a warp
+// reads eight runs of 64 bytes of a partial.
 __global__ void __launch_bounds__(256) prefill_merge_kernel(const __grid_constant__ MergeParams p) {
     grid_dep_wait();  // the partials come from the prefill launch before this one
     const int hpc = p.heads_per_cta;
@@ -741,7 +771,7 @@ __global__ void __launch_bounds__(256) prefill_merge_kernel(const __grid_constan
             if (i0 + k < ns) {
                 const int64_t b = pblk(i0 + k);
                 ml[k] = __ldcg(reinterpret_cast<const float2 *>(p.part_ml + (b * kTileQ + r) * 2));
-                o[k] = __ldcg(reinterpret_cast<const float4 *>(p.part_o + ((b * 4 + c4) * kTileQ + r) * 32) + j4);
+                o[k] = __ldcg(reinterpret_cast<const float4 *>(p.part_o) + (b * (kHeadDim / 4) + c4 * 8 + j4) * kTileQ + r);
             } else {
                 ml[k] = make_float2(-INFINITY, 0.f);
                 o[k] = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -76,7 +76,7 @@ struct PrefillParamsT {
     int32_t heads_per_cta;  // 2 when the group has >= 2 heads, else 1
     float scale_log2;       // scale * log2(e)
     int32_t *err;
-    float *part_o;          // [n_part, heads_per_cta, 4 chunks, 128 rows, 32]
+    float *part_o;          // [n_part, heads_per_cta, 32 chunks, 128 rows, 4]
     float *part_ml;         // [n_part, heads_per_cta, 128 rows, 2]
     int32_t n_ctas;         // CTAs running prefill items
     uint16_t cta_begin[kMaxPrefillCtas + 1];  // CTA c runs work[cta_begin[c] .. cta_begin[c + 1])
