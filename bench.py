@@ -48,7 +48,7 @@ HEADLINE_WORKLOAD = ("MBT 16384 low pressure: 25,000-token prompt planned into c
 # sha256 of the kernel's device code it was measured on (reported only while
 # that code is unchanged).
 PREFILL_TRAFFIC = {
-    "8cec327c70337d26": 84111872 + 26717952,   # ncu capture of one (16384, p=0) layer
+    "d112e467d647f486": 83995648 + 27335936,   # ncu capture of one (16384, p=0) layer
 }
 
 

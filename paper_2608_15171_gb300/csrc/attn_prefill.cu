@@ -17,22 +17,21 @@
 // no room apart) Q K^T had to wait for the P V that reads P, and the chain
 // softmax -> P V -> Q K^T set the pace: 4340 cycles a KV tile of both Q
 // tiles (2048 of them MMA), the two softmax warpgroups held apart by a turn
-// barrier.  Now they overlap, 3100-3300 cycles a KV tile, and what is left
-// is the loop Q K^T (540 in issue) -> S seen (250) -> S read out (200) ->
-// next Q K^T (165-300) twice a tile, with P V in its gaps.
+// barrier.  Now they overlap.  The MMA and TMA warps run their loops as
+// whole warps and only issue under elect_one(): with a loop of lane 0 the
+// operands of every MMA and copy went through ordinary registers, and 8
+// MMAs with their commits and the loop around them took the issuing thread
+// about 1400 cycles instead of the tensor core's 512.
 // Warp roles (512 threads, four warpgroups):
 //   warps 0-3   TMA producers: warps 0/1 fetch pages 0-3 / 4-7 of each K
 //               tile (3-stage ring), warps 2/3 those of each V tile (2
 //               stages), through the block table.  One issuing thread moves
 //               only ~7 B/clk of small TMA boxes on GB300, so every tile is
 //               fetched by two threads.
-//   warp 4      Q K^T issuer (one thread): S = Q_t K^T (A = Q in shared
+//   warp 4      Q K^T issuer: S = Q_t K^T (A = Q in shared
 //               memory) for t = 0, 1, as soon as S has been read out.
-//   warp 5      P V issuer (one thread): O_t += P_t V (A = P in TMEM).  A
-//               batch goes out behind the Q K^T batch after the next one
-//               (see there).  One thread for both took 4400 cycles a KV
-//               tile: a thread that issues MMAs is held up until the tensor
-//               core has taken them, so its waits and commits are gaps.
+//   warp 5      P V issuer: O_t += P_t V (A = P in TMEM).  A batch goes
+//               out behind the Q K^T batch after the next one (see there).
 //   warp 6      Q loader: Q_t of the next item once the last Q K^T of the
 //               current item on tile t has completed.
 //   warps 8-11  softmax for tile 0, warps 12-15 for tile 1: each thread owns
@@ -44,9 +43,11 @@
 // with setmaxnreg.  The running max is only raised (and O rescaled in TMEM)
 // when it grows by more than 2^8; until then the stale max keeps every
 // exponent <= 2^8, and the final O / l is exact either way.
-// (16384 tokens over an empty prefix, 16/2 heads: 922 us before, 735 now;
-// 8616 over 16384: 1221 -> 985; the ratio shrinks by a few percent in a long
-// run, where the faster kernel draws the clock down.)
+// 16384 tokens over an empty prefix, 16/2 heads, 1.0996 TFLOP of causal work:
+// 922 us with P over S, 735 with S apart, 620-640 issued by whole warps (565 us,
+// 1.95 PFLOP/s, in the first 50 ms of a run; after that the GPU lowers its
+// clock, as under a cuBLAS GEMM).  What bounds it now is the tensor core, and
+// in a long run the power it draws.
 // The host plan may cut a long (query tile, head slot) unit into pieces on
 // consecutive CTAs (stream-K): each piece writes its partial (m, l, O) to the
 // workspace, and prefill_merge_kernel, launched after this kernel, combines
@@ -291,7 +292,8 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
     const uint32_t sb = (raw_s + 1023u) & ~1023u;  // 1024-aligned for the 128-byte swizzle
     uint8_t *const sg = smem_raw + (sb - raw_s);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (uniform)
     const int hpc = p.heads_per_cta;
     // this CTA's items, in order
     const int w_beg = p.cta_begin[cta], w_end = p.cta_begin[cta + 1];
@@ -333,7 +335,7 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(sg + kOffTmem);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(sg + kOffTmem), 0);
     // the set-up above overlaps the previous kernel of the stream; global
     // memory (KV pages, Q, block tables, outputs) only after it has completed
     grid_dep_wait();
@@ -343,39 +345,31 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
         // The rings run on across item boundaries: tile g of this CTA (over
         // all its items) goes to stage g % depth.
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsSmall));
-        if (lane == 0 && w_beg < w_end) {
+        if (w_beg < w_end) {
             const bool is_v = warp >= 2;
-            const int pg_lo = (warp & 1) * (kPagesPerTile / 2);  // this thread's pages of each tile
+            const int pg_lo = (warp & 1) * (kPagesPerTile / 2);  // this warp's pages of each tile
             const int ns = is_v ? kNV : kNK;
             const CUtensorMap *tm = is_v ? &tm_v : &tm_k;
             const uint32_t ring = sb + (is_v ? kOffV : kOffK);
             const int full0 = is_v ? B_VFULL : B_KFULL, empty0 = is_v ? B_VEMPTY : B_KEMPTY;
+            const int pg = pg_lo + (lane & 3);  // lane i (mod 4) looks after page pg_lo + i
             // page ids of the next tile are loaded while the current one is issued
-            int ids[kPagesPerTile / 2];
-            auto load_ids = [&](const ItemView &v, int jj) {
+            int id = 0;
+            auto load_id = [&](const ItemView &v, int jj) {
                 const int j = v.kt0 + jj;
-                const int np = pages_in(v.ctx_len, j);
-#pragma unroll
-                for (int i = 0; i < kPagesPerTile / 2; ++i)
-                    ids[i] = (pg_lo + i < np) ? __ldg(v.table + j * kPagesPerTile + pg_lo + i) : 0;
+                id = pg < pages_in(v.ctx_len, j) ? __ldg(v.table + j * kPagesPerTile + pg) : 0;
             };
             int w = w_beg, jj = 0;
             ItemView cur = item_view(p, w);
-            load_ids(cur, 0);
+            load_id(cur, 0);
             for (int g = 0;; ++g) {
-                const int j = cur.kt0 + jj;
                 const int s = g % ns;
-                const int np = max(0, min(kPagesPerTile / 2, pages_in(cur.ctx_len, j) - pg_lo));
-                int rows[kPagesPerTile / 2];
-#pragma unroll
-                for (int i = 0; i < kPagesPerTile / 2; ++i) {
-                    int blk = ids[i];
-                    if (i < np && (blk < 0 || blk >= p.num_blocks)) {
-                        report_error(p.err, PPAS_DEVERR_BAD_INDEX);
-                        blk = 0;  // keep the barrier's byte count consistent
-                    }
-                    rows[i] = (blk * p.n_kv_heads + cur.kvh) * kPage;
+                const int np = max(0, min(kPagesPerTile / 2, pages_in(cur.ctx_len, cur.kt0 + jj) - pg_lo));
+                if (pg - pg_lo < np && (id < 0 || id >= p.num_blocks)) {
+                    if (lane < 4) report_error(p.err, PPAS_DEVERR_BAD_INDEX);
+                    id = 0;  // keep the barrier's byte count consistent
                 }
+                const int row = (id * p.n_kv_heads + cur.kvh) * kPage;
                 // the next tile: this item's, else the next item's first
                 int jn = jj + 1, wn = w;
                 if (jn == cur.n_kt) {
@@ -384,18 +378,26 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                 }
                 const bool more = wn < w_end;
                 const ItemView nxt = (more && wn != w) ? item_view(p, wn) : cur;
-                if (more) load_ids(nxt, jn);
-                if (g >= ns && !mbar_wait(bar(empty0 + s), ((g / ns) & 1) ^ 1, p.err)) {
+                if (more) load_id(nxt, jn);
+                if (g >= ns && !mbar_wait_warp(bar(empty0 + s), ((g / ns) & 1) ^ 1, p.err)) {
                     *abort_flag = 1;
                     break;
                 }
-                const uint32_t b = bar(full0 + s);
-                mbar_expect_tx(b, static_cast<uint32_t>(np) * 2 * kBox);
-                const uint32_t dst = ring + s * kTileBytes + pg_lo * kBox;
-                for (int i = 0; i < np; ++i) {
-                    tma_load_2d(dst + i * kBox, tm, 0, rows[i], b);
-                    tma_load_2d(dst + kHalf + i * kBox, tm, 64, rows[i], b);
+                int rows[kPagesPerTile / 2];
+#pragma unroll
+                for (int i = 0; i < kPagesPerTile / 2; ++i) rows[i] = __shfl_sync(0xffffffffu, row, i);
+                if (elect_one()) {
+                    const uint32_t b = bar(full0 + s);
+                    mbar_expect_tx(b, static_cast<uint32_t>(np) * 2 * kBox);
+                    const uint32_t dst = ring + s * kTileBytes + pg_lo * kBox;
+#pragma unroll
+                    for (int i = 0; i < kPagesPerTile / 2; ++i)
+                        if (i < np) {
+                            tma_load_2d(dst + i * kBox, tm, 0, rows[i], b);
+                            tma_load_2d(dst + kHalf + i * kBox, tm, 64, rows[i], b);
+                        }
                 }
+                __syncwarp();
                 if (!more) break;
                 w = wn;
                 jj = jn;
@@ -404,7 +406,7 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
         }
     } else if (warp < kSoftmaxWarp0) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsSmall));
-        if (warp == kMmaWarp && lane == 0 && w_beg < w_end) {
+        if (warp == kMmaWarp && w_beg < w_end) {
             // -------------------------------------------------------- Q K^T issuer
             // descriptors are built once; advancing one operand by b bytes
             // adds b >> 4 to the start-address field (no carry: < 256 KB)
@@ -417,32 +419,36 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                 const ItemView v = item_view(p, w);
                 for (int jj = 0; ok && jj < v.n_kt; ++jj, ++g) {
                     const int sk = g % kNK;
-                    if (!mbar_wait(bar(B_KFULL + sk), (g / kNK) & 1, p.err)) { ok = false; break; }
+                    if (!mbar_wait_warp(bar(B_KFULL + sk), (g / kNK) & 1, p.err)) { ok = false; break; }
                     const uint64_t dk = dk0 + ((sk * kTileBytes) >> 4);
                     for (int t = 0; t < hpc; ++t, ++n) {
-                        if (jj == 0 && !mbar_wait(bar(B_Q + t), i & 1, p.err)) { ok = false; break; }
+                        if (jj == 0 && !mbar_wait_warp(bar(B_Q + t), i & 1, p.err)) { ok = false; break; }
                         // the S columns, once the softmax before has read them out
-                        if (n >= 1 && !mbar_wait(bar(B_SFREE), (n - 1) & 1, p.err)) { ok = false; break; }
+                        if (n >= 1 && !mbar_wait_warp(bar(B_SFREE), (n - 1) & 1, p.err)) { ok = false; break; }
                         tc_fence_after();
                         const uint64_t dq = dq0 + ((t * kTileBytes) >> 4);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int kk = 0; kk < 8; ++kk) {
-                            const uint32_t o = (kk >> 2) * kHalf + (kk & 3) * 32;
-                            umma_bf16(tmem + kColS, dq + (o >> 4), dk + (o >> 4), kIdescQK, kk > 0 ? 1u : 0u);
+                            for (int kk = 0; kk < 8; ++kk) {
+                                const uint32_t o = (kk >> 2) * kHalf + (kk & 3) * 32;
+                                umma_bf16(tmem + kColS, dq + (o >> 4), dk + (o >> 4), kIdescQK, kk > 0 ? 1u : 0u);
+                            }
+                            umma_commit(bar(B_SFULL + t));
+                            mbar_arrive(bar(B_QKI + (n & 3)));  // P V (n - hpc) may follow
+                            if (t == hpc - 1) umma_commit(bar(B_KEMPTY + sk));
+                            // the item's last Q K^T frees Q_t for the next item
+                            if (jj == v.n_kt - 1) umma_commit(bar(B_QEMPTY + t));
                         }
-                        umma_commit(bar(B_SFULL + t));
-                        mbar_arrive(bar(B_QKI + (n & 3)));  // P V (n - hpc) may follow
-                        if (t == hpc - 1) umma_commit(bar(B_KEMPTY + sk));
-                        // the item's last Q K^T frees Q_t for the next item
-                        if (jj == v.n_kt - 1) umma_commit(bar(B_QEMPTY + t));
+                        __syncwarp();
                     }
                 }
             }
             if (!ok) *abort_flag = 1;
             // every MMA issued so far completes before TMEM is released
-            umma_commit(bar(B_DRAIN));
+            if (elect_one()) umma_commit(bar(B_DRAIN));
+            __syncwarp();
             mbar_wait(bar(B_DRAIN), 0, p.err);
-        } else if (warp == kMmaWarp + 1 && lane == 0 && w_beg < w_end) {
+        } else if (warp == kMmaWarp + 1 && w_beg < w_end) {
             // -------------------------------------------------------- P V issuer
             const uint64_t dv0 = smem_desc_sw128(sb + kOffV, kHalf, 1024);
             bool ok = true;
@@ -451,47 +457,52 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                 const ItemView v = item_view(p, w);
                 for (int jj = 0; ok && jj < v.n_kt; ++jj, ++g) {
                     const int sv = g % kNV;
-                    if (!mbar_wait(bar(B_VFULL + sv), (g / kNV) & 1, p.err)) { ok = false; break; }
+                    if (!mbar_wait_warp(bar(B_VFULL + sv), (g / kNV) & 1, p.err)) { ok = false; break; }
                     const uint64_t dv = dv0 + ((sv * kTileBytes) >> 4);
                     const int chunks = pages_in(v.ctx_len, v.kt0 + jj);
                     for (int t = 0; t < hpc; ++t) {
-                        if (!mbar_wait(bar(B_PFULL + t), g & 1, p.err)) { ok = false; break; }
+                        if (!mbar_wait_warp(bar(B_PFULL + t), g & 1, p.err)) { ok = false; break; }
                         // P V (n) goes out behind Q K^T (n + hpc): P V (n) and
                         // the read-out of S (n + hpc - 1), which lets that
                         // Q K^T start, are ready at about the same time, and
                         // the tensor core would work on both batches in turn
-                        // while the softmax waits for S (809 us without this
-                        // rule, 788 with it).  Not for the last KV tile of an
-                        // item: the Q K^T after it may wait for the epilogues.
+                        // while the softmax waits for S (16384 tokens: 695 us
+                        // without this rule, 623 with it).  Not for the last KV
+                        // tile of an item: the Q K^T after it may wait for the
+                        // epilogues.
                         // Q K^T runs at most n + 2 hpc ahead of P V (n) (the
                         // softmax stores P (n + hpc) only after P V (n)), so
                         // four barriers keep its phases apart.
                         if (jj + 1 < v.n_kt) {
                             const int gate = (g + 1) * hpc + t;
-                            if (!mbar_wait(bar(B_QKI + (gate & 3)), (gate >> 2) & 1, p.err)) { ok = false; break; }
+                            if (!mbar_wait_warp(bar(B_QKI + (gate & 3)), (gate >> 2) & 1, p.err)) { ok = false; break; }
                         }
                         tc_fence_after();
                         // O_t += P_t V(j), P_t from TMEM; the item's first tile overwrites O_t
                         const uint32_t d_p = tmem + kColP + t * 64, d_o = tmem + kColO + t * 128;
-                        if (chunks == kPagesPerTile) {
+                        if (elect_one()) {
+                            if (chunks == kPagesPerTile) {
 #pragma unroll
-                            for (int kk = 0; kk < kPagesPerTile; ++kk)
-                                umma_bf16_ts(d_o, d_p + kk * 8, dv + ((kk * 2048) >> 4), kIdescPV,
-                                             (jj > 0 || kk > 0) ? 1u : 0u);
-                        } else {
-                            for (int kk = 0; kk < chunks; ++kk)
-                                umma_bf16_ts(d_o, d_p + kk * 8, dv + ((kk * 2048) >> 4), kIdescPV,
-                                             (jj > 0 || kk > 0) ? 1u : 0u);
+                                for (int kk = 0; kk < kPagesPerTile; ++kk)
+                                    umma_bf16_ts(d_o, d_p + kk * 8, dv + ((kk * 2048) >> 4), kIdescPV,
+                                                 (jj > 0 || kk > 0) ? 1u : 0u);
+                            } else {
+                                for (int kk = 0; kk < chunks; ++kk)
+                                    umma_bf16_ts(d_o, d_p + kk * 8, dv + ((kk * 2048) >> 4), kIdescPV,
+                                                 (jj > 0 || kk > 0) ? 1u : 0u);
+                            }
+                            umma_commit(bar(B_ODONE + t));
+                            if (t == hpc - 1) umma_commit(bar(B_VEMPTY + sv));
                         }
-                        umma_commit(bar(B_ODONE + t));
-                        if (t == hpc - 1) umma_commit(bar(B_VEMPTY + sv));
+                        __syncwarp();
                     }
                 }
             }
             if (!ok) *abort_flag = 1;
-            umma_commit(bar(B_DRAIN));
+            if (elect_one()) umma_commit(bar(B_DRAIN));
+            __syncwarp();
             mbar_wait(bar(B_DRAIN), 0, p.err);
-        } else if (warp == kQWarp && lane == 0) {
+        } else if (warp == kQWarp) {
             // -------------------------------------------------------- Q loader
             // Q tile t of item i is loaded once the last Q K^T of item i-1 on
             // that tile has completed.
@@ -501,13 +512,16 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                 const int h0 = wk.slot * hpc;
                 bool ok = true;
                 for (int t = 0; t < hpc; ++t) {
-                    if (i > 0 && !mbar_wait(bar(B_QEMPTY + t), (i - 1) & 1, p.err)) {
+                    if (i > 0 && !mbar_wait_warp(bar(B_QEMPTY + t), (i - 1) & 1, p.err)) {
                         ok = false;
                         break;
                     }
-                    mbar_expect_tx(bar(B_Q + t), kTileBytes);
-                    tma_load_3d(sb + kOffQ + t * kTileBytes, &tm_q, 0, h0 + t, qrow, bar(B_Q + t));
-                    tma_load_3d(sb + kOffQ + t * kTileBytes + kHalf, &tm_q, 64, h0 + t, qrow, bar(B_Q + t));
+                    if (elect_one()) {
+                        mbar_expect_tx(bar(B_Q + t), kTileBytes);
+                        tma_load_3d(sb + kOffQ + t * kTileBytes, &tm_q, 0, h0 + t, qrow, bar(B_Q + t));
+                        tma_load_3d(sb + kOffQ + t * kTileBytes + kHalf, &tm_q, 64, h0 + t, qrow, bar(B_Q + t));
+                    }
+                    __syncwarp();
                 }
                 if (!ok) {
                     *abort_flag = 1;
