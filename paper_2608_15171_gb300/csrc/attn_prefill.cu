@@ -249,12 +249,6 @@ __device__ __forceinline__ void store_rows(void *dst, bool fp32, int64_t stride,
             *reinterpret_cast<uint4 *>(d + i * stride) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
 }
 
-// mbar_wait() by a whole warp: one vote when the phase is complete already
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int32_t *err) {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
-}
-
 // The parts of a work item each role needs (read from the kernel parameters).
 struct ItemView {
     const int32_t *table;  // the sequence's block-table row

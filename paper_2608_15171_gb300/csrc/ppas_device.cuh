@@ -77,6 +77,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t
     }
 }
 
+// mbar_wait() by a whole warp: one vote when the phase is complete already
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int32_t *err) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
+}
+
 // ---------------------------------------------------------------- named barriers
 // bar.sync / bar.arrive on a named barrier (0 is __syncthreads); n counts
 // threads (a multiple of 32) and every warp taking part executes it as a
