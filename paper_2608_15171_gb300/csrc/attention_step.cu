@@ -896,16 +896,21 @@ extern "C" ppas_status ppas_gateup_swiglu(const void *x, const void *w_packed, v
     if (hidden < 64 || hidden % 64 || inter < 128 || inter % 128) return PPAS_ERR_UNSUPPORTED;
     if (n_tokens == 0) return PPAS_OK;
     if (!x || !w_packed || !y || !aligned16(x) || !aligned16(w_packed) || !aligned16(y)) return PPAS_ERR_INVALID_ARG;
-    CUtensorMap tm_x, tm_w;
-    if (!encode_bf16_2d(&tm_x, x, static_cast<uint64_t>(hidden), static_cast<uint64_t>(n_tokens), 64, 128) ||
-        !encode_bf16_2d(&tm_w, w_packed, static_cast<uint64_t>(hidden), 2ull * inter, 64, 256))
-        return PPAS_ERR_CUDA;
     GateUpParams gp;
     gp.y = static_cast<__nv_bfloat16 *>(y);
     gp.n_tokens = n_tokens;
     gp.hidden = hidden;
     gp.inter = inter;
     gp.err = d_err_flag;
+    const bool few = n_tokens <= kFewTokens;
+    CUtensorMap tm_x, tm_w;
+    if (!encode_bf16_2d(&tm_x, x, static_cast<uint64_t>(hidden), static_cast<uint64_t>(n_tokens), 64,
+                        few ? static_cast<uint32_t>((n_tokens + 15) & ~15) : 128) ||
+        !encode_bf16_2d(&tm_w, w_packed, static_cast<uint64_t>(hidden), 2ull * inter, 64, few ? 64 : 256))
+        return PPAS_ERR_CUDA;
+    if (few)
+        return launch_gateup_few(tm_x, tm_w, gp, static_cast<cudaStream_t>(stream)) == cudaSuccess ? PPAS_OK
+                                                                                                   : PPAS_ERR_CUDA;
     const int64_t tiles = static_cast<int64_t>((n_tokens + 127) / 128) * (inter / 128);
     const int grid = static_cast<int>(std::min<int64_t>(tiles, device_sm_count()));
     return launch_gateup(tm_x, tm_w, gp, grid, static_cast<cudaStream_t>(stream)) == cudaSuccess ? PPAS_OK

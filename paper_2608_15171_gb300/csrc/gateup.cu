@@ -66,6 +66,18 @@ __device__ __forceinline__ void tile_mn(int t, int m_blocks, int n_blocks, int &
     mb = grp * kGroupM + rem % gm;
 }
 
+__device__ __forceinline__ void tmem_ld16_sync(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+          "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+
 __device__ __forceinline__ void tmem_ld32_wait(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
     asm volatile(
@@ -244,6 +256,162 @@ __global__ void __launch_bounds__(kGThreads, 1)
     }
 }
 
+// ---------------------------------------------------------------- few tokens
+// At most kFewTokens tokens (a decode iteration): the projection is bound by
+// streaming the weights, so the operands change sides.  A = weights, 64 gate
+// rows and the 64 up rows of the same features as one M128 tile; B = all the
+// tokens (N = tokens rounded up to 16).  One CTA per 64 features, two CTAs to
+// an SM, so that at inter = 11008 all 172 CTAs stream at once (the kernel
+// above has 86 tiles and pads the tokens to 128 rows of MMA work).
+// 192 threads: warp 0 TMA, warp 1 MMA, warps 2-5 epilogue: gate and up
+// accumulators of a feature lie 64 TMEM lanes apart, so both go through shared
+// memory (the ring, once the last MMA has completed).
+// Hidden 2048, inter 11008 (90 MB of weights): see launch_gateup_few.
+constexpr int kFF = 64;  // features per CTA
+constexpr uint32_t kFewA = 128 * kGK * 2;  // weight tile of a K block: 16 KB
+constexpr uint32_t kFewRing = 112640;      // ring bytes at most: two CTAs share an SM
+constexpr int kFewMaxStages = 6;
+
+// accumulator columns to allocate: a power of two, at least 32
+__host__ __device__ constexpr int few_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : 128; }
+__host__ __device__ constexpr uint32_t few_stage(int n) { return kFewA + static_cast<uint32_t>(n) * kGK * 2; }
+__host__ __device__ constexpr int few_stages(int n) {
+    return static_cast<int>(kFewRing / few_stage(n)) < kFewMaxStages ? static_cast<int>(kFewRing / few_stage(n))
+                                                                     : kFewMaxStages;
+}
+static_assert(few_stages(kFewTokens) >= 3, "ring depth");
+static_assert(kFewTokens * 128 * 4 <= few_stages(kFewTokens) * few_stage(kFewTokens), "epilogue buffer in the ring");
+
+__global__ void __launch_bounds__(kGThreads, 2)
+    gateup_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
+                      const __grid_constant__ GateUpParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bars[2 * kFewMaxStages + 1];
+    __shared__ uint32_t tmem_base;
+    __shared__ int abort_word;
+    const uint32_t raw_s = smem_u32(smem_raw);
+    const uint32_t sb = (raw_s + 1023u) & ~1023u;
+    float *const buf = reinterpret_cast<float *>(smem_raw + (sb - raw_s));  // [128 rows][n] after the MMAs
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (uniform)
+    auto full = [&](int s) { return smem_u32(bars) + 8u * static_cast<uint32_t>(s); };
+    auto empty = [&](int s) { return smem_u32(bars) + 8u * static_cast<uint32_t>(kFewMaxStages + s); };
+    const uint32_t done = smem_u32(bars) + 8u * (2 * kFewMaxStages);
+    volatile int *abort_flag = &abort_word;
+
+    const int n = (p.n_tokens + 15) & ~15;
+    const uint32_t stage = few_stage(n);
+    const int stages = few_stages(n);
+    const int k_blocks = p.hidden / kGK;
+    const int f0 = blockIdx.x * kFF;                       // first feature
+    const int w_row = (f0 / 128) * 256 + (f0 % 128);       // its gate row in the packed weight; up: + 128
+
+    if (warp == 1) {
+        tmem_alloc(smem_u32(&tmem_base), few_cols(n));
+        tmem_relinquish();
+    }
+    if (tid == 0) {
+        for (int s = 0; s < stages; ++s) {
+            mbar_init(full(s), 1);
+            mbar_init(empty(s), 1);
+        }
+        mbar_init(done, 1);
+        *abort_flag = 0;
+        fence_mbar_init();
+        prefetch_tmap(&tm_x);
+        prefetch_tmap(&tm_w);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *const_cast<volatile uint32_t *>(&tmem_base), 0);
+    // the set-up above overlaps the kernel before this one on the stream
+    grid_dep_wait();
+    grid_dep_launch();
+
+    if (warp == 0) {
+        for (int kb = 0, s = 0, round = 0; kb < k_blocks; ++kb) {
+            if (round > 0 && !mbar_wait_warp(empty(s), (round - 1) & 1, p.err)) {
+                *abort_flag = 1;
+                break;
+            }
+            if (elect_one()) {
+                const uint32_t dst = sb + s * stage;
+                mbar_expect_tx(full(s), stage);
+                tma_load_2d(dst, &tm_w, kb * kGK, w_row, full(s));
+                tma_load_2d(dst + kFewA / 2, &tm_w, kb * kGK, w_row + 128, full(s));
+                tma_load_2d(dst + kFewA, &tm_x, kb * kGK, 0, full(s));
+            }
+            __syncwarp();
+            if (++s == stages) {
+                s = 0;
+                ++round;
+            }
+        }
+    } else if (warp == 1) {
+        const uint64_t da0 = smem_desc_sw128(sb, 16, 1024);
+        const uint64_t db0 = smem_desc_sw128(sb + kFewA, 16, 1024);
+        const uint32_t idesc = idesc_bf16_f32(128, 16, false, false) +
+                               (static_cast<uint32_t>((n - 16) >> 3) << 17);  // N = n
+        bool ok = true;
+        for (int kb = 0, s = 0, round = 0; kb < k_blocks; ++kb) {
+            if (!mbar_wait_warp(full(s), round & 1, p.err)) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            const uint64_t da = da0 + ((s * stage) >> 4), db = db0 + ((s * stage) >> 4);
+            if (elect_one()) {
+#pragma unroll
+                for (int kk = 0; kk < kGK / 16; ++kk)
+                    umma_bf16(tmem, da + kk * 2, db + kk * 2, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                umma_commit(empty(s));
+            }
+            __syncwarp();
+            if (++s == stages) {
+                s = 0;
+                ++round;
+            }
+        }
+        if (!ok) *abort_flag = 1;
+        // every MMA issued so far has completed once `done` is set
+        if (elect_one()) umma_commit(done);
+        __syncwarp();
+        mbar_wait(done, 0, p.err);
+    } else {
+        const int wq = warp & 3;  // TMEM lane quarter: rows 0-63 gate, 64-127 up
+        const bool ok = mbar_wait_warp(done, 0, p.err) && !__any_sync(0xffffffffu, *abort_flag);
+        tc_fence_after();
+        const uint32_t t_lane = tmem + (static_cast<uint32_t>(wq * 32) << 16);
+        if (ok)
+            for (int c = 0; c < n; c += 16) {
+                uint32_t v[16];
+                tmem_ld16_sync(t_lane + c, v);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) buf[(c + i) * 128 + wq * 32 + lane] = __uint_as_float(v[i]);
+            }
+        nbar_sync(1, 128);
+        if (ok) {
+            // one warp per token: a lane's two features
+            for (int t = wq; t < p.n_tokens; t += 4) {
+                const float2 g = *reinterpret_cast<const float2 *>(buf + t * 128 + 2 * lane);
+                const float2 u = *reinterpret_cast<const float2 *>(buf + t * 128 + 64 + 2 * lane);
+                const float y0 = __fdividef(g.x, 1.f + __expf(-g.x)) * u.x;
+                const float y1 = __fdividef(g.y, 1.f + __expf(-g.y)) * u.y;
+                *reinterpret_cast<uint32_t *>(p.y + static_cast<int64_t>(t) * p.inter + f0 + 2 * lane) =
+                    pack_bf16x2(y0, y1);
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, few_cols(n));
+    }
+}
+
 // W [2I, H] (gate rows, then up rows) -> packed: block j of 256 rows holds
 // gate rows 128j .. 128j+127 then up rows I+128j .. I+128j+127.
 __global__ void gateup_pack_kernel(const uint4 *__restrict__ w, uint4 *__restrict__ wp, int hidden, int inter) {
@@ -266,6 +434,24 @@ cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, cons
     if (e != cudaSuccess) return e;
     gateup_swiglu_kernel<<<grid, kGThreads, kSmemG, st>>>(tm_x, tm_w, p);
     return cudaGetLastError();
+}
+
+// Times on one GB300, the kernel above before and this one now (hidden 2048,
+// inter 11008, 90 MB of weights): 1 token 26.5 -> 18.1 us, 8: 25.3 -> 17.8,
+// 32: 22.3 -> 16.9, 64: 22.7 -> 18.6, 128: 23.4 -> 20.5 (the copy bandwidth
+// takes 13.4); hidden 4096, inter 14336 (235 MB), 4 tokens: 55.1 -> 37.7.  Past
+// 128 tokens every CTA would read more of x than of the weights, and the
+// ring would fall below three stages: those calls stay with the kernel above
+// (129 tokens: 31.9).
+cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p,
+                              cudaStream_t st) {
+    static std::atomic<uint64_t> smem_set{0};
+    const cudaError_t e =
+        ensure_smem_limit(gateup_few_kernel, static_cast<int>(kFewRing + 1024), smem_set);
+    if (e != cudaSuccess) return e;
+    const int n = (p.n_tokens + 15) & ~15;
+    PdlLaunch l(dim3(p.inter / kFF), dim3(kGThreads), few_stages(n) * few_stage(n) + 1024, st);
+    return cudaLaunchKernelEx(&l.cfg, gateup_few_kernel, tm_x, tm_w, p);
 }
 
 cudaError_t launch_gateup_pack(const void *w, void *wp, int hidden, int inter, cudaStream_t st) {

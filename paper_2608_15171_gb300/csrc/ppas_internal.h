@@ -274,6 +274,11 @@ bool encode_bf16_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t
 
 cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p, int grid,
                           cudaStream_t st);
+// calls of at most this many tokens take the weight-streaming kernel
+constexpr int kFewTokens = 128;
+// tm_x: box of (n_tokens rounded up to 16) rows; tm_w: box of 64 rows
+cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p,
+                              cudaStream_t st);
 cudaError_t launch_gateup_pack(const void *w, void *wp, int hidden, int inter, cudaStream_t st);
 
 // launch configuration with programmatic stream serialization: the kernel

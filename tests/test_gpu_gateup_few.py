@@ -1,0 +1,51 @@
+"""The weight-streaming gate-up kernel (calls of at most 128 tokens) at the
+edges of its range: one token, around each multiple of 16 that changes the
+MMA's N, the largest call it takes and the first one past it; the smallest
+K and feature counts, and K longer than the ring.  Every element against the
+float64 oracle, and the rows after the last token untouched."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import mlp
+from test_gpu_gateup import _check, _inputs, ppas  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 33, 64, 65, 127, 128, 129])
+@pytest.mark.parametrize("H,I", [(64, 128), (1024, 384)])
+def test_every_element_and_nothing_past_the_tokens(ppas, T, H, I):  # noqa: F811
+    x, w = _inputs(T, H, I, seed=3 * T + H)
+    wp = torch.empty_like(w)
+    ppas.ppas_gateup_pack(w, wp, H, I)
+    y = torch.full((T + 3, I), 7.0, dtype=torch.bfloat16, device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ppas.ppas_gateup_swiglu(x, wp, y, T, H, I, err)
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    assert bool((y[T:] == 7.0).all())
+    _check(y[:T].float().cpu().numpy(), mlp.gate_up(x.float().cpu().numpy(), w.float().cpu().numpy()),
+           f"T={T} H={H} I={I}")
+
+
+def test_back_to_back_calls_on_each_others_output(ppas):  # noqa: F811
+    """Each call reads what the call before wrote (the kernel sets up while
+    its predecessor still runs): a chain of calls equals the same chain with
+    a wait after each."""
+    T, H = 24, 256
+    x, w = _inputs(T, H, H, seed=11)
+    wp = torch.empty_like(w)
+    ppas.ppas_gateup_pack(w, wp, H, H)
+    got = []
+    for wait in (True, False):
+        a = x.clone()
+        for _ in range(6):
+            b = torch.empty_like(a)
+            ppas.ppas_gateup_swiglu(a, wp, b, T, H, H)
+            if wait:
+                torch.cuda.synchronize()
+            a = b
+        torch.cuda.synchronize()
+        got.append(a.float().cpu().numpy())
+    assert np.array_equal(got[0], got[1])
