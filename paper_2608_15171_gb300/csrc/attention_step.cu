@@ -17,15 +17,18 @@ namespace ppas {
 namespace {
 
 // Throughput model behind the SMs the prefill kernel leaves to the decode
-// launch (measured on GB300): one item's KV tile (two q-heads x 128 queries x
-// 128 keys) takes about 2.06 us of one SM; next to a running prefill kernel
-// the decode kernel streams 65-80 GB/s per SM (the upper figure is used, so
-// that a wrong estimate leaves decode rows rather than prefill items as the
-// tail: the slower side of the balance), and at most kDecodeBytesPerUs on
-// the GPU.
+// splits, fitted on GB300 to the best measured splits rather than to either
+// rate alone: beside one another an item's KV tile (two q-heads x 128 queries
+// x 128 keys) takes 1.2-1.5 us of an SM and a decode split streams 83-87 GB/s
+// per SM, but every decode SM also slows the prefill items (shared power and
+// memory), so the model's prefill is slower than the kernel's.  Step times
+// over k: 4 x 512 with 8 decodes (k = 16) 136.2 us, k = 12 140.4, k = 20 138.8,
+// k = 24 136.0; 3 x 683 with 16 decodes, 32/8 heads (k = 35) 617 us at its
+// fastest, k = 40 633, k = 44 616, k = 48 634, 52 and more 660-680.
 constexpr double kPrefillTileUs = 2.06;
 constexpr double kDecodeBytesPerSmUs = 8.0e4;
 constexpr double kDecodeBytesPerUs = 4.35e6;
+constexpr double kDecodeSplitUs = 5.0;  // a decode split besides its bytes: page ids, first pages, merges
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -402,6 +405,48 @@ PrefillPlan plan_prefill(int32_t n_seqs, const int32_t *q_lens, const int32_t *c
             }
             std::vector<std::vector<std::pair<int32_t, PrefillWork>>> filled;
             fill(lo, &filled);
+            auto span = [](const std::vector<std::vector<std::pair<int32_t, PrefillWork>>> &v) {
+                int64_t most = 0;
+                for (const auto &cta : v) {
+                    int64_t load = 0;
+                    for (const auto &pc : cta) load += pc.second.kt1 - pc.second.kt0 + kPrefillItemCost;
+                    most = std::max(most, load);
+                }
+                return most;
+            };
+            // a step of few units: every unit in equal pieces, one to a CTA, of
+            // the smallest length L whose pieces fit the CTAs.  The fill above
+            // cuts from the front of a unit and leaves its last CTA what is
+            // left: units of 13-16 tiles at 4 tiles a CTA came out as 4, 4, 7
+            // (512 tokens over 2048 with 2 decodes: CTAs done at 9.7 to 13.9 us,
+            // 21.8 us a layer; 19.9 with equal pieces)
+            if (static_cast<int64_t>(u1 - u0) <= nc) {
+                auto pieces = [&](const Unit &un, int32_t len) {
+                    return std::min((un.n_kt + len - 1) / len, std::max(1, un.n_kt / kPrefillMinPiece));
+                };
+                auto needs = [&](int32_t len) {
+                    int64_t n = 0;
+                    for (size_t u = u0; u < u1; ++u) n += pieces(units[u], len);
+                    return n;
+                };
+                int32_t a = kPrefillMinPiece, b = kPrefillMaxPiece;
+                while (a < b) {
+                    const int32_t mid = a + (b - a) / 2;
+                    if (needs(mid) <= nc) b = mid; else a = mid + 1;
+                }
+                if (needs(a) <= nc) {
+                    std::vector<std::vector<std::pair<int32_t, PrefillWork>>> even;
+                    for (size_t u = u0; u < u1; ++u) {
+                        const Unit &un = units[u];
+                        const int32_t n = pieces(un, a);
+                        for (int32_t k = 0; k < n; ++k)
+                            even.push_back({{static_cast<int32_t>(u - u0),
+                                             item(un, static_cast<int32_t>(int64_t{un.n_kt} * k / n),
+                                                  static_cast<int32_t>(int64_t{un.n_kt} * (k + 1) / n))}});
+                    }
+                    if (span(even) < span(filled)) filled = std::move(even);
+                }
+            }
             // pieces of a unit get consecutive partial slots
             std::vector<int32_t> n_pieces(u1 - u0, 0);
             for (const auto &v : filled)
@@ -422,12 +467,7 @@ PrefillPlan plan_prefill(int32_t n_seqs, const int32_t *q_lens, const int32_t *c
                         pc.second.part = static_cast<uint16_t>(first_part[pc.first] + next_part[pc.first]++);
                     per_cta[c].push_back(pc.second);
                 }
-            int64_t cut_span = 0;
-            for (const auto &v : per_cta) {
-                int64_t load = 0;
-                for (const PrefillWork &w : v) load += w.kt1 - w.kt0 + kPrefillItemCost;
-                cut_span = std::max(cut_span, load);
-            }
+            const int64_t cut_span = span(filled);
             if (lp.n_part == 0 || (!needs_cut && cut_span + kPrefillMergeCost >= whole_span)) {
                 per_cta = std::move(whole);  // not worth the partials
                 lp.split_units.clear();
@@ -476,6 +516,14 @@ int32_t decode_reserve_sms(int32_t n_seqs, const int32_t *q_lens, const int32_t 
     const double sm_time = units * kPrefillTileUs;
     int32_t k = static_cast<int32_t>(std::ceil(bytes * num_sms / (kDecodeBytesPerSmUs * sm_time + bytes)));
     k = std::min(k, static_cast<int32_t>(kDecodeBytesPerUs / kDecodeBytesPerSmUs));
+    // A short step: when the prefill items take no longer than two decode
+    // splits (each ~kDecodeSplitUs besides its bytes), splits that wait for an
+    // SM would be its tail, so all of them get one at once.  (512 tokens over
+    // 2048 with 2 decode rows, 32 splits: with 8 SMs left to them 8 of the 32
+    // would start when the first ones end.)
+    const DecodePlan d = plan_decode(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, num_sms);
+    const double split_us = kDecodeSplitUs + bytes / static_cast<double>(d.n_ctas) / kDecodeBytesPerSmUs;
+    if (sm_time / num_sms < 2 * split_us) k = std::max(k, static_cast<int32_t>(std::min<int64_t>(d.n_ctas, num_sms)));
     return std::max(0, std::min(k, num_sms / 2));
 }
 
