@@ -23,6 +23,13 @@
 // tickets never need clearing before a launch; the kernel is launched with
 // programmatic stream serialization and touches global memory only after
 // grid_dep_wait().
+// A step of one row is a chain of latencies once its 26 MB have streamed (at
+// 5.8 of its 13.3 us, per-CTA timestamps), so the tail is kept short: the
+// ticket is claimed before the merges by a reduction nobody waits for, one
+// thread fences instead of all, the heads of a merge are independent
+// loads, and the last CTA has up to 20 partials in flight.  One row x 25k,
+// 16/2 heads, append + attention: 14.3 -> 13.0 us a layer.  (Claiming at entry
+// cost the page loop 1 %: 96 rows of 17-4100 tokens 270.8 -> 274.5 us.)
 #include <math.h>
 
 #include "ppas_device.cuh"
@@ -269,6 +276,21 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
         for (int i = consumed; i < min(consumed + kDecodeStages, my_count); ++i)
             mbar_wait(bar(i % kDecodeStages), (i / kDecodeStages) & 1, nullptr);
 
+    // CTAs per thread-block cluster: 1 unless the launch groups the splits of
+    // a (row, kv-head) into clusters (steps of decode rows only)
+    const uint32_t nct = kPartial ? 1u : cluster_nctarank();
+    const uint32_t crank = nct > 1 ? cluster_ctarank() : 0u;
+
+    // The splits of a (row, kv-head) count their arrivals in a ticket =
+    // (tag << 16) | arrivals.  Tags grow from launch to launch, so a maximum
+    // turns a word left by an earlier launch (or reset to 0) into this
+    // launch's tag with no arrivals, and leaves a word this launch already
+    // owns alone.  The split claims the word here, without waiting for an
+    // answer, and adds its arrival (one atomic) when its partial is written.
+    unsigned long long *const ctr = p.counters + lo * p.n_kv_heads + kvh;
+    const unsigned long long ticket0 = p.launch_tag << 16;
+    if (tid == 0 && row.n_splits > 1 && crank == 0) atomicMax(ctr, ticket0);
+
     l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
     l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
 
@@ -286,13 +308,9 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
         for (int n = 0; n < 16; ++n) *reinterpret_cast<float2 *>(dst + n * 8 + 2 * c) = make_float2(o[n][0], o[n][1]);
     }
     decode_cta_sync<kPartial>();
-    // CTAs per thread-block cluster: 1 unless the launch groups the splits of
-    // a (row, kv-head) into clusters (steps of decode rows only)
-    const uint32_t nct = kPartial ? 1u : cluster_nctarank();
     // (in a cluster an aborted CTA carries on to the cluster barrier below)
     if (nct == 1 && *abort_flag) return;
     // rank 0's slot for this CTA's partial (cluster launches only)
-    const uint32_t crank = nct > 1 ? cluster_ctarank() : 0u;
     const uint32_t recv = sb + kOffClusterRecv;
     const uint32_t slot_o = nct > 1 ? dsmem_addr(recv + crank * (kMaxGroup * kHeadDim * 4), 0) : 0u;
     const uint32_t slot_ml =
@@ -300,40 +318,54 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
     if (nct > 1) cluster_wait();  // every CTA of the cluster has started (its arrive at entry)
 
     // thread -> (head-dim column, first head); the CTA's threads cover
-    // kDecodeThreads / 128 heads at a time
+    // kDecodeThreads / 128 heads at a time, all of a group's in one round of
+    // independent loads
     const int t = tid & (kHeadDim - 1);
-    const int hstep = kDecodeThreads / kHeadDim;
-    for (int hh = tid / kHeadDim; hh < g; hh += hstep) {
-        float M = -INFINITY;
+    constexpr int hstep = kDecodeThreads / kHeadDim, kHeads = kMaxGroup / hstep;
+    const int h0 = tid / kHeadDim;
+    float Mh[kHeads], Lh[kHeads], Oh[kHeads];
 #pragma unroll
-        for (int w = 0; w < kDecodeWarps; ++w) M = fmaxf(M, cm[w * kMaxGroup + hh]);
-        float L = 0.f, O = 0.f;
+    for (int i = 0; i < kHeads; ++i) {
+        const int hh = h0 + i * hstep;
+        if (hh >= g) break;
+        float m[kDecodeWarps];
+        Mh[i] = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < kDecodeWarps; ++w) {
+            m[w] = cm[w * kMaxGroup + hh];
+            Mh[i] = fmaxf(Mh[i], m[w]);
+        }
+        Lh[i] = Oh[i] = 0.f;
 #pragma unroll
         for (int w = 0; w < kDecodeWarps; ++w) {
             // a warp without keys (or a split past its row's pages, which a
             // cluster plan may hold) has m = -inf and weight 0
-            const float m = cm[w * kMaxGroup + hh];
-            const float f = m == -INFINITY ? 0.f : ex2(m - M);
-            L += f * cl[w * kMaxGroup + hh];
-            O += f * co[(w * kMaxGroup + hh) * kHeadDim + t];
+            const float f = m[w] == -INFINITY ? 0.f : ex2(m[w] - Mh[i]);
+            Lh[i] += f * cl[w * kMaxGroup + hh];
+            Oh[i] += f * co[(w * kMaxGroup + hh) * kHeadDim + t];
         }
+    }
+#pragma unroll
+    for (int i = 0; i < kHeads; ++i) {
+        const int hh = h0 + i * hstep;
+        if (hh >= g) break;
         const int head = kvh * g + hh;
         if (row.n_splits == 1) {
             const int64_t oi = (static_cast<int64_t>(row.q_row) * p.n_q_heads + head) * kHeadDim + t;
-            if (p.out_fp32) static_cast<float *>(p.out)[oi] = O / L;
-            else static_cast<__nv_bfloat16 *>(p.out)[oi] = __float2bfloat16_rn(O / L);
+            if (p.out_fp32) static_cast<float *>(p.out)[oi] = Oh[i] / Lh[i];
+            else static_cast<__nv_bfloat16 *>(p.out)[oi] = __float2bfloat16_rn(Oh[i] / Lh[i]);
         } else if (nct > 1) {
-            dsmem_st_f32(slot_o + static_cast<uint32_t>(hh * kHeadDim + t) * 4u, O);
+            dsmem_st_f32(slot_o + static_cast<uint32_t>(hh * kHeadDim + t) * 4u, Oh[i]);
             if (t == 0) {
-                dsmem_st_f32(slot_ml + static_cast<uint32_t>(hh * 2) * 4u, M);
-                dsmem_st_f32(slot_ml + static_cast<uint32_t>(hh * 2 + 1) * 4u, L);
+                dsmem_st_f32(slot_ml + static_cast<uint32_t>(hh * 2) * 4u, Mh[i]);
+                dsmem_st_f32(slot_ml + static_cast<uint32_t>(hh * 2 + 1) * 4u, Lh[i]);
             }
         } else {
             const int64_t pi = static_cast<int64_t>(row.part_base + sp) * p.n_q_heads + head;
-            p.part_o[pi * kHeadDim + t] = O;
+            p.part_o[pi * kHeadDim + t] = Oh[i];
             if (t == 0) {
-                p.part_ml[pi * 2] = M;
-                p.part_ml[pi * 2 + 1] = L;
+                p.part_ml[pi * 2] = Mh[i];
+                p.part_ml[pi * 2 + 1] = Lh[i];
             }
         }
     }
@@ -351,22 +383,36 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
             if (crank != 0) return;
             const float *ro = reinterpret_cast<const float *>(sg + kOffClusterRecv);
             const float *rml = ro + kMaxCluster * kMaxGroup * kHeadDim;
-            for (int hh = tid / kHeadDim; hh < g; hh += hstep) {
-                float M = -INFINITY;
-                for (uint32_t r = 0; r < nct; ++r) M = fmaxf(M, rml[(r * kMaxGroup + hh) * 2]);
-                float L = 0.f, O = 0.f;
-                for (uint32_t r = 0; r < nct; ++r) {
-                    const float m = rml[(r * kMaxGroup + hh) * 2];
-                    const float f = m == -INFINITY ? 0.f : ex2(m - M);
-                    L += f * rml[(r * kMaxGroup + hh) * 2 + 1];
-                    O += f * ro[(r * kMaxGroup + hh) * kHeadDim + t];
+#pragma unroll
+            for (int i = 0; i < kHeads; ++i) {
+                const int hh = h0 + i * hstep;
+                if (hh >= g) break;
+                float m[kMaxCluster];
+                Mh[i] = -INFINITY;
+#pragma unroll
+                for (int r = 0; r < kMaxCluster; ++r) {
+                    m[r] = r < static_cast<int>(nct) ? rml[(r * kMaxGroup + hh) * 2] : -INFINITY;
+                    Mh[i] = fmaxf(Mh[i], m[r]);
                 }
+                Lh[i] = Oh[i] = 0.f;
+#pragma unroll
+                for (int r = 0; r < kMaxCluster; ++r)
+                    if (m[r] != -INFINITY) {
+                        const float f = ex2(m[r] - Mh[i]);
+                        Lh[i] += f * rml[(r * kMaxGroup + hh) * 2 + 1];
+                        Oh[i] += f * ro[(r * kMaxGroup + hh) * kHeadDim + t];
+                    }
+            }
+#pragma unroll
+            for (int i = 0; i < kHeads; ++i) {
+                const int hh = h0 + i * hstep;
+                if (hh >= g) break;
                 const int64_t pi =
                     static_cast<int64_t>(row.part_base + sp / static_cast<int>(nct)) * p.n_q_heads + kvh * g + hh;
-                p.part_o[pi * kHeadDim + t] = O;
+                p.part_o[pi * kHeadDim + t] = Oh[i];
                 if (t == 0) {
-                    p.part_ml[pi * 2] = M;
-                    p.part_ml[pi * 2 + 1] = L;
+                    p.part_ml[pi * 2] = Mh[i];
+                    p.part_ml[pi * 2 + 1] = Lh[i];
                 }
             }
             n_parts = row.n_splits / static_cast<int>(nct);
@@ -374,33 +420,33 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
     }
 
     // ---- the last CTA of this (row, kv-head) merges every split
-    __threadfence();
     decode_cta_sync<kPartial>();
     __shared__ int s_last;
     if (tid == 0) {
-        // ticket = (tag << 16) | arrivals.  Tags grow from launch to launch, so
-        // atomicMax turns a word left by an earlier launch (or reset to 0)
-        // into this launch's tag with no arrivals, and leaves a word this
-        // launch already owns alone; only a word with a larger tag (memory
-        // nothing of this process wrote) is claimed by compare-and-swap.
-        // Then every split adds its arrival: two atomics, no retries.
-        unsigned long long *ctr = p.counters + lo * p.n_kv_heads + kvh;
-        const unsigned long long mine = p.launch_tag << 16;
-        unsigned long long cur = atomicMax(ctr, mine);
-        for (int it = 0; (cur >> 16) > p.launch_tag && it < (1 << 20); ++it) {
-            const unsigned long long got = atomicCAS(ctr, cur, mine);
-            cur = got == cur ? mine : got;
+        __threadfence();  // the whole CTA's partials (ordered before this by the barrier), then the arrival
+        unsigned long long old = atomicAdd(ctr, 1ull);
+        int prev = (old >> 16) == p.launch_tag ? static_cast<int>(old & 0xFFFFull) : -1;
+        // a word with a larger tag (memory nothing of this process wrote):
+        // the splits that met it count themselves again, from one of them on
+        unsigned long long cur = old + 1;
+        for (int it = 0; prev < 0 && it < (1 << 20); ++it) {
+            if ((cur >> 16) == p.launch_tag) {
+                old = atomicAdd(ctr, 1ull);
+                prev = static_cast<int>(old & 0xFFFFull);
+            } else {
+                const unsigned long long got = atomicCAS(ctr, cur, ticket0 + 1);
+                if (got == cur) prev = 0;
+                cur = got;
+            }
         }
-        const unsigned long long old = atomicAdd(ctr, 1ull);
-        const int prev = (old >> 16) == p.launch_tag ? static_cast<int>(old & 0xFFFFull) : -1;
         if (prev < 0) report_error(p.err, PPAS_DEVERR_TIMEOUT);  // the word was never claimed
         s_last = (prev == n_parts - 1);
         if (s_last) *ctr = 0;  // also ready for a replay with the same tag (a captured graph)
+        __threadfence();
     }
     decode_cta_sync<kPartial>();
     if (!s_last) return;
-    __threadfence();
-    // Warp hh merges head hh on its own (lane: 4 columns).  The first 16
+    // Warp hh merges head hh on its own (lane: 4 columns).  The first kBatch
     // splits' O go out before the weights are known, so their latency hides
     // that of the (m, l) round; the weights w = 2^(m - M) stay in a
     // shared-memory row of the warp (the rings are free), 1 / L is applied
@@ -411,9 +457,10 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
     const int head = kvh * g + hh;
     const float4 *po = reinterpret_cast<const float4 *>(p.part_o) + c4;
     auto part_index = [&](int s_) { return static_cast<int64_t>(row.part_base + s_) * p.n_q_heads + head; };
-    float4 ov[16];
+    constexpr int kBatch = 20;  // a one-row step in clusters has 18 or 19 partials: one round
+    float4 ov[kBatch];
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
+    for (int k = 0; k < kBatch; ++k)
         ov[k] = k < ns ? __ldcg(po + part_index(k) * (kHeadDim / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
     float *wm = reinterpret_cast<float *>(sg) + hh * 2 * kMaxDecodeSplitsPerRow;  // [ns] m, then w
     float *wl = wm + kMaxDecodeSplitsPerRow;                                     // [ns] l
@@ -437,14 +484,14 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
     for (int o_ = 16; o_ >= 1; o_ >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o_);
     __syncwarp();
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < ns; s0 += 16) {
+    for (int s0 = 0; s0 < ns; s0 += kBatch) {
         if (s0 > 0) {
 #pragma unroll
-            for (int k = 0; k < 16; ++k)
+            for (int k = 0; k < kBatch; ++k)
                 ov[k] = s0 + k < ns ? __ldcg(po + part_index(s0 + k) * (kHeadDim / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
+        for (int k = 0; k < kBatch; ++k) {
             const float f = s0 + k < ns ? wm[s0 + k] : 0.f;
             acc = make_float4(acc.x + f * ov[k].x, acc.y + f * ov[k].y, acc.z + f * ov[k].z, acc.w + f * ov[k].w);
         }
