@@ -5,25 +5,33 @@
 //
 // The weights are packed once (gateup_pack_kernel) so that every 256-row
 // block holds 128 gate rows followed by the 128 up rows of the same
-// features.  One output tile is 128 tokens x 128 features: a single
-// M128 x N256 accumulator whose left half is the gate product and right half
-// the up product, so the epilogue combines them without leaving the SM and
-// the [T, 2I] intermediate never reaches HBM.
+// features.  One output tile is 256 tokens x 128 features, worked by a pair of
+// CTAs (cta_group::2): M 256 (128 tokens in each CTA) x N 256 (gate products
+// left, up products right), so the epilogue combines them without leaving
+// the SM and the [T, 2I] intermediate never reaches HBM.  Each CTA of the pair
+// loads its own tokens and half of the weight rows: 32 KB of L2 traffic for 64
+// columns of K and 512 tensor cycles.  A CTA by itself with the same 128 x 256
+// share needs 48 KB, 96 B/clk on every SM, which L2 does not deliver (2056
+// tokens, hidden 2048, inter 11008: 118.1 us; the pairs take 108.8, 16,384
+// tokens 815 -> 740 us in a short run, 896 -> 838 at the power limit of a long
+// one; 1024 tokens 66.0 -> 55.8, 256 33.2 -> 25.0).
 //
 // Persistent kernel, one CTA per SM, 192 threads:
-//   warp 0      TMA producer: X tile (128 x 64) and W tile (256 x 64) per
-//               64-wide K block, 128-byte swizzle, 4-stage ring
-//   warp 1      allocates TMEM, issues the MMAs (4 x K16 per K block) into one
-//               of two 256-column accumulators
+//   warp 0      TMA producer: X tile (128 x 64) and W tile (128 x 64) per
+//               64-wide K block, 128-byte swizzle, 6-stage ring; both CTAs'
+//               bytes are counted by the leader's barrier
+//   warp 1      allocates TMEM; the leader's issues the pair's MMAs (4 x K16 per
+//               K block) into one of two 256-column accumulators, and its
+//               commits release the ring and fill the accumulators in both CTAs
 //   warps 2-5   epilogue: each thread owns one token row (its TMEM lane),
 //               reads 32 gate and 32 up columns at a time, writes bf16
 // The producer and MMA warps run their loops as whole warps and only issue
 // under elect_one(), which keeps descriptors and addresses in uniform
-// registers (2056 tokens, hidden 2048, inter 11008: 121.0 -> 118.0 us against
-// loops of lane 0; 16,384 tokens: 898 -> 883).
-// Tiles are visited in groups of 32 M blocks with the M block fastest, so
-// the CTAs running at one time share a few weight tiles and keep a few MB of
-// X tiles hot in L2.
+// registers (2-2.5 % against loops of lane 0).
+// Tiles are visited in groups of 16 M blocks with the M block fastest, so
+// the pairs running at one time share a few weight tiles and keep a few MB of
+// X tiles hot in L2 (groups of 8: 2056 tokens 114.5 against 112.9 us).
+// Calls of at most kFewTokens tokens take another kernel, below.
 #include <algorithm>
 
 #include "ppas_device.cuh"
@@ -32,13 +40,13 @@
 namespace ppas {
 namespace {
 
-constexpr int kGM = 128;   // tokens per tile
+constexpr int kGM = 256;   // tokens per tile: 128 in each CTA of a pair
 constexpr int kGN = 256;   // accumulator columns: 128 gate + 128 up
 constexpr int kGK = 64;    // K per stage (128 bytes of bf16: one swizzle row)
-constexpr int kGStages = 4;
-constexpr int kGroupM = 32;  // M blocks per raster group
-constexpr uint32_t kABytes = kGM * kGK * 2;  // 16 KB
-constexpr uint32_t kBBytes = kGN * kGK * 2;  // 32 KB
+constexpr int kGStages = 6;
+constexpr int kGroupM = 16;  // M blocks per raster group
+constexpr uint32_t kABytes = kGM / 2 * kGK * 2;  // 16 KB in each CTA
+constexpr uint32_t kBBytes = kGN / 2 * kGK * 2;  // 16 KB in each CTA
 constexpr uint32_t kStage = kABytes + kBBytes;
 constexpr uint32_t kOffBarG = kGStages * kStage;
 enum : int {
@@ -55,7 +63,12 @@ constexpr uint32_t kSmemG = kOffBarG + 256 + 1024;  // + alignment slack
 static_assert(kOffAbortG + 4 <= kOffBarG + 256, "barrier area");
 static_assert(kSmemG <= 232448, "shared memory per CTA");
 constexpr int kGThreads = 192;
-constexpr uint32_t kIdescG = idesc_bf16_f32(kGM, kGN, false, false);  // A, B both K-major
+
+// One item of a pair: a tile, or one of `cut` equal column slices of it.
+struct GateUpItem {
+    int mb, nb;     // m block, n block (128 features)
+    int f0, width;  // the slice's first feature within the block, and its features
+};
 
 // tile index -> (m block, n block), M fastest within groups of kGroupM
 __device__ __forceinline__ void tile_mn(int t, int m_blocks, int n_blocks, int &mb, int &nb) {
@@ -96,11 +109,22 @@ __device__ __forceinline__ void tmem_ld32_wait(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// item t of the launch: the first n_full are whole tiles, the others slices
+__device__ __forceinline__ GateUpItem gateup_item(const GateUpParams &p, int t, int m_blocks, int n_blocks) {
+    GateUpItem it;
+    const int u = t - p.n_full;
+    const int tile = u < 0 ? t : p.n_full + u / p.cut;
+    tile_mn(tile, m_blocks, n_blocks, it.mb, it.nb);
+    it.width = u < 0 ? kGN / 2 : kGN / 2 / p.cut;
+    it.f0 = u < 0 ? 0 : (u % p.cut) * it.width;
+    return it;
+}
+
 }  // namespace
 
-__global__ void __launch_bounds__(kGThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
     gateup_swiglu_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
-                         const __grid_constant__ GateUpParams p) {
+                         const __grid_constant__ CUtensorMap tm_cut, const __grid_constant__ GateUpParams p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_s = smem_u32(smem_raw);
     const uint32_t sb = (raw_s + 1023u) & ~1023u;
@@ -112,12 +136,14 @@ __global__ void __launch_bounds__(kGThreads, 1)
 
     const int m_blocks = (p.n_tokens + kGM - 1) / kGM;
     const int n_blocks = p.inter / (kGN / 2);
-    const int n_tiles = m_blocks * n_blocks;
+    const int n_items = p.n_items;
     const int k_blocks = p.hidden / kGK;
+    const uint32_t rank = cluster_ctarank();  // 0: the pair's leader
+    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
     if (warp == 1) {
-        tmem_alloc(sb + kOffTmemG, 512);
-        tmem_relinquish();
+        tmem_alloc_pair(sb + kOffTmemG, 512);
+        tmem_relinquish_pair();
     }
     if (tid == 0) {
         for (int s = 0; s < kGStages; ++s) {
@@ -126,108 +152,122 @@ __global__ void __launch_bounds__(kGThreads, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar(G_ACCFULL + b), 1);
-            mbar_init(bar(G_ACCEMPTY + b), 4);  // one arrive per epilogue warp
+            mbar_init(bar(G_ACCEMPTY + b), 8);  // one arrive per epilogue warp of the pair
         }
         mbar_init(bar(G_DRAIN), 1);
         *abort_flag = 0;
         fence_mbar_init();
         prefetch_tmap(&tm_x);
         prefetch_tmap(&tm_w);
+        prefetch_tmap(&tm_cut);
     }
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    cluster_sync_all();  // both CTAs' barriers and TMEM are there
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(sg + kOffTmemG), 0);
+    // the set-up above overlaps the kernel before this one on the stream
+    grid_dep_wait();
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
+        // each CTA loads its 128 tokens and its half of the weight rows (rank
+        // 0: the gate rows, rank 1: the up rows); all of a stage's bytes
+        // are counted by the leader's barrier
         int q = 0;  // K blocks issued by this CTA
-        for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-            int mb, nb;
-            tile_mn(t, m_blocks, n_blocks, mb, nb);
-            bool ok = true;
+        bool ok = true;
+        for (int t = pair; ok && t < n_items; t += n_pairs) {
+            const GateUpItem item = gateup_item(p, t, m_blocks, n_blocks);
+            const int x_row = item.mb * kGM + static_cast<int>(rank) * (kGM / 2);
+            const int w_row = item.nb * kGN + static_cast<int>(rank) * (kGN / 2) + item.f0;
+            const CUtensorMap *tw = t < p.n_full ? &tm_w : &tm_cut;
+            const uint32_t bytes = kABytes + static_cast<uint32_t>(item.width) * kGK * 2;
             for (int kb = 0; kb < k_blocks; ++kb, ++q) {
                 const int s = q % kGStages;
                 if (q >= kGStages && !mbar_wait_warp(bar(G_EMPTY + s), ((q / kGStages) & 1) ^ 1, p.err)) {
                     ok = false;
                     break;
                 }
+                const uint32_t full = dsmem_addr(bar(G_FULL + s), 0);
                 if (elect_one()) {
                     const uint32_t dst = sb + s * kStage;
-                    mbar_expect_tx(bar(G_FULL + s), kStage);
-                    tma_load_2d(dst, &tm_x, kb * kGK, mb * kGM, bar(G_FULL + s));
-                    tma_load_2d(dst + kABytes, &tm_w, kb * kGK, nb * kGN, bar(G_FULL + s));
+                    if (rank == 0) mbar_expect_tx(bar(G_FULL + s), 2 * bytes);
+                    tma_load_2d_pair(dst, &tm_x, kb * kGK, x_row, full);
+                    tma_load_2d_pair(dst + kABytes, tw, kb * kGK, w_row, full);
                 }
                 __syncwarp();
             }
-            if (!ok || __any_sync(0xffffffffu, *abort_flag)) {
-                *abort_flag = 1;
-                break;
-            }
+            if (__any_sync(0xffffffffu, *abort_flag)) ok = false;
         }
+        // the leader's last releases of the ring have reached this CTA before it leaves
+        for (int j = max(0, q - kGStages); ok && j < q; ++j)
+            ok = mbar_wait_warp(bar(G_EMPTY + j % kGStages), (j / kGStages) & 1, p.err);
+        if (!ok) *abort_flag = 1;
+        // every MMA of the pair has completed, and this CTA has been told
+        mbar_wait_warp(bar(G_DRAIN), 0, p.err);
     } else if (warp == 1) {
-        // ---------------------------------------------------------------- MMA issuer
-        const uint64_t da0 = smem_desc_sw128(sb, 16, 1024);
-        const uint64_t db0 = smem_desc_sw128(sb + kABytes, 16, 1024);
-        int q = 0, it = 0;
-        bool ok = true;
-        for (int t = blockIdx.x; ok && t < n_tiles; t += gridDim.x, ++it) {
-            const int buf = it & 1;
-            const uint32_t d = tmem + buf * kGN;
-            // the epilogue has drained this accumulator (two tiles ago)
-            if (it >= 2 && !mbar_wait_warp(bar(G_ACCEMPTY + buf), ((it >> 1) & 1) ^ 1, p.err)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            for (int kb = 0; kb < k_blocks; ++kb, ++q) {
-                const int s = q % kGStages;
-                if (!mbar_wait_warp(bar(G_FULL + s), (q / kGStages) & 1, p.err)) {
+        // ---------------------------------------------------------------- MMA issuer (the leader's)
+        if (rank == 0) {
+            const uint64_t da0 = smem_desc_sw128(sb, 16, 1024);
+            const uint64_t db0 = smem_desc_sw128(sb + kABytes, 16, 1024);
+            int q = 0, it = 0;
+            bool ok = true;
+            for (int t = pair; ok && t < n_items; t += n_pairs, ++it) {
+                const int buf = it & 1;
+                const uint32_t d = tmem + buf * kGN;
+                const uint32_t idesc = t < p.n_full ? idesc_bf16_f32(kGM, kGN, false, false)
+                                                    : idesc_bf16_f32(kGM, kGN / p.cut, false, false);
+                // both epilogues have drained this accumulator (two tiles ago)
+                if (it >= 2 && !mbar_wait_warp(bar(G_ACCEMPTY + buf), ((it >> 1) & 1) ^ 1, p.err)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint64_t da = da0 + ((s * kStage) >> 4), db = db0 + ((s * kStage) >> 4);
-                if (elect_one()) {
+                for (int kb = 0; kb < k_blocks; ++kb, ++q) {
+                    const int s = q % kGStages;
+                    if (!mbar_wait_warp(bar(G_FULL + s), (q / kGStages) & 1, p.err)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint64_t da = da0 + ((s * kStage) >> 4), db = db0 + ((s * kStage) >> 4);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < kGK / 16; ++kk)
-                        umma_bf16(d, da + (kk * 2), db + (kk * 2), kIdescG, (kb > 0 || kk > 0) ? 1u : 0u);
-                    umma_commit(bar(G_EMPTY + s));
-                    if (kb == k_blocks - 1) umma_commit(bar(G_ACCFULL + buf));
+                        for (int kk = 0; kk < kGK / 16; ++kk)
+                            umma_bf16_pair(d, da + (kk * 2), db + (kk * 2), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                        umma_commit_pair(bar(G_EMPTY + s));
+                        if (kb == k_blocks - 1) umma_commit_pair(bar(G_ACCFULL + buf));
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
+            if (!ok) *abort_flag = 1;
+            if (elect_one()) umma_commit_pair(bar(G_DRAIN));
         }
-        if (!ok) *abort_flag = 1;
-        if (elect_one()) umma_commit(bar(G_DRAIN));
-        __syncwarp();
-        mbar_wait(bar(G_DRAIN), 0, p.err);
     } else {
         // ---------------------------------------------------------------- epilogue
         const int wq = warp & 3;  // TMEM lane quarter of this warp
-        const int r = wq * 32 + lane;
         const uint32_t t_lane = tmem + (static_cast<uint32_t>(wq * 32) << 16);
         int it = 0;
-        for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
+        for (int t = pair; t < n_items; t += n_pairs, ++it) {
             const int buf = it & 1;
-            const bool ok = __all_sync(0xffffffffu, !*abort_flag &&
-                                                        mbar_wait(bar(G_ACCFULL + buf), (it >> 1) & 1, p.err));
+            const bool ok = mbar_wait_warp(bar(G_ACCFULL + buf), (it >> 1) & 1, p.err) &&
+                            !__any_sync(0xffffffffu, *abort_flag);
             if (!ok) {
                 *abort_flag = 1;
                 break;
             }
             tc_fence_after();
-            int mb, nb;
-            tile_mn(t, m_blocks, n_blocks, mb, nb);
-            const int row = mb * kGM + r;
-            __nv_bfloat16 *out = p.y + static_cast<int64_t>(row) * p.inter + nb * (kGN / 2);
+            const GateUpItem item = gateup_item(p, t, m_blocks, n_blocks);
+            const int row0 = item.mb * kGM + static_cast<int>(rank) * (kGM / 2) + wq * 32;  // the warp's first token
+            __nv_bfloat16 *out = p.y + static_cast<int64_t>(row0) * p.inter + item.nb * (kGN / 2) + item.f0;
 #pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < item.width / 32; ++c) {
                 float gv[32], uv[32];
                 tmem_ld32_wait(t_lane + buf * kGN + c * 32, gv);
-                tmem_ld32_wait(t_lane + buf * kGN + 128 + c * 32, uv);
-                if (row < p.n_tokens) {
-                    uint4 *dst = reinterpret_cast<uint4 *>(out + c * 32);
+                tmem_ld32_wait(t_lane + buf * kGN + item.width + c * 32, uv);
+                if (row0 + lane < p.n_tokens) {
+                    uint4 *dst = reinterpret_cast<uint4 *>(out + static_cast<int64_t>(lane) * p.inter + c * 32);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         uint32_t w4[4];
@@ -244,15 +284,18 @@ __global__ void __launch_bounds__(kGThreads, 1)
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(G_ACCEMPTY + buf));
+            if (lane == 0) mbar_arrive_cluster(dsmem_addr(bar(G_ACCEMPTY + buf), 0));
         }
     }
 
+    // neither CTA frees its TMEM or leaves while the other's MMAs, copies or
+    // arrivals may still reach it
     tc_fence_before();
-    __syncthreads();
+    __syncwarp();
+    cluster_sync_all();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, 512);
+        tmem_dealloc_pair(tmem, 512);
     }
 }
 
@@ -261,8 +304,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
 // streaming the weights, so the operands change sides.  A = weights, 64 gate
 // rows and the 64 up rows of the same features as one M128 tile; B = all the
 // tokens (N = tokens rounded up to 16).  One CTA per 64 features, two CTAs to
-// an SM, so that at inter = 11008 all 172 CTAs stream at once (the kernel
-// above has 86 tiles and pads the tokens to 128 rows of MMA work).
+// an SM, so that at inter = 11008 all 172 CTAs stream at once (tiles of 128
+// tokens x 128 features are 86, and pad the tokens to 128 rows of MMA work).
 // 192 threads: warp 0 TMA, warp 1 MMA, warps 2-5 epilogue: gate and up
 // accumulators of a feature lie 64 TMEM lanes apart, so both go through shared
 // memory (the ring, once the last MMA has completed).
@@ -427,22 +470,22 @@ __global__ void gateup_pack_kernel(const uint4 *__restrict__ w, uint4 *__restric
     }
 }
 
-cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p, int grid,
-                          cudaStream_t st) {
+cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const CUtensorMap &tm_cut,
+                          const GateUpParams &p, int pairs, cudaStream_t st) {
     static std::atomic<uint64_t> smem_set{0};
     const cudaError_t e = ensure_smem_limit(gateup_swiglu_kernel, static_cast<int>(kSmemG), smem_set);
     if (e != cudaSuccess) return e;
-    gateup_swiglu_kernel<<<grid, kGThreads, kSmemG, st>>>(tm_x, tm_w, p);
-    return cudaGetLastError();
+    PdlLaunch l(dim3(2 * pairs), dim3(kGThreads), kSmemG, st);
+    return cudaLaunchKernelEx(&l.cfg, gateup_swiglu_kernel, tm_x, tm_w, tm_cut, p);
 }
 
-// Times on one GB300, the kernel above before and this one now (hidden 2048,
+// Times on one GB300, with 128-token tiles before and now (hidden 2048,
 // inter 11008, 90 MB of weights): 1 token 26.5 -> 18.1 us, 8: 25.3 -> 17.8,
 // 32: 22.3 -> 16.9, 64: 22.7 -> 18.6, 128: 23.4 -> 20.5 (the copy bandwidth
 // takes 13.4); hidden 4096, inter 14336 (235 MB), 4 tokens: 55.1 -> 37.7.  Past
 // 128 tokens every CTA would read more of x than of the weights, and the
-// ring would fall below three stages: those calls stay with the kernel above
-// (129 tokens: 31.9).
+// ring would fall below three stages: those calls take the kernel above (129
+// tokens: 24.2).
 cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p,
                               cudaStream_t st) {
     static std::atomic<uint64_t> smem_set{0};

@@ -265,15 +265,26 @@ struct GateUpParams {
     int32_t hidden;    // multiple of 64
     int32_t inter;     // multiple of 128
     int32_t *err;
+    // a launch of CTA pairs: the first n_full of its n_items are whole tiles
+    // (256 tokens x 128 features), the rest slices of 128 / cut features of the
+    // tiles after them
+    int32_t n_full, cut, n_items;
 };
+struct GateUpPlan {
+    int32_t pairs, n_full, cut, n_items;
+};
+// the items of n_tokens x inter over max_pairs CTA pairs
+GateUpPlan plan_gateup(int32_t n_tokens, int32_t inter, int32_t max_pairs);
 
 // 2D bf16 row-major tensor [outer, inner] with a (box_inner x box_outer) box,
 // 128-byte swizzle (box_inner * 2 bytes must be 128)
 bool encode_bf16_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint32_t box_inner,
                     uint32_t box_outer);
 
-cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p, int grid,
-                          cudaStream_t st);
+// pairs: CTA pairs (one item at a time each); tm_x, tm_w: boxes of 128 rows;
+// tm_cut: of 128 / p.cut
+cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const CUtensorMap &tm_cut,
+                          const GateUpParams &p, int pairs, cudaStream_t st);
 // calls of at most this many tokens take the weight-streaming kernel
 constexpr int kFewTokens = 128;
 // tm_x: box of (n_tokens rounded up to 16) rows; tm_w: box of 64 rows

@@ -1,8 +1,9 @@
-"""The weight-streaming gate-up kernel (calls of at most 128 tokens) at the
-edges of its range: one token, around each multiple of 16 that changes the
+"""The gate-up kernels at the edges of their ranges.  The weight-streaming one
+(calls of at most 128 tokens): one token, around each multiple of 16 that changes the
 MMA's N, the largest call it takes and the first one past it; the smallest
 K and feature counts, and K longer than the ring.  Every element against the
-float64 oracle, and the rows after the last token untouched."""
+float64 oracle, and the rows after the last token untouched.  The CTA-pair
+one: see there."""
 import numpy as np
 import pytest
 import torch
@@ -22,6 +23,32 @@ def test_every_element_and_nothing_past_the_tokens(ppas, T, H, I):  # noqa: F811
     y = torch.full((T + 3, I), 7.0, dtype=torch.bfloat16, device="cuda")
     err = torch.zeros(1, dtype=torch.int32, device="cuda")
     ppas.ppas_gateup_swiglu(x, wp, y, T, H, I, err)
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    assert bool((y[T:] == 7.0).all())
+    _check(y[:T].float().cpu().numpy(), mlp.gate_up(x.float().cpu().numpy(), w.float().cpu().numpy()),
+           f"T={T} H={H} I={I}")
+
+
+@pytest.mark.parametrize("T,H,I", [
+    (129, 64, 128 * 40),    # 40 tiles: one round of whole tiles
+    (200, 128, 128 * 30),   # 30 tiles: halves
+    (256, 64, 128 * 19),    # 19 tiles: quarters
+    (257, 192, 128),        # 2 tiles, the second of one token
+    (513, 64, 128 * 27),    # 81 tiles: a round of whole tiles, then 5 in quarters
+    (400, 64, 128 * 55),    # 110 tiles: whole, then 34 in halves
+])
+def test_pair_tiles_and_slices_of_the_last_round(ppas, T, H, I):  # noqa: F811
+    """Calls of the CTA-pair kernel whose last round is whole, halved or
+    quartered (on 76 pairs), ragged in tokens, K shorter than the ring; and
+    the rows after the last token untouched."""
+    x, w = _inputs(T, H, I, seed=T + I)
+    wp = torch.empty_like(w)
+    ppas.ppas_gateup_pack(w, wp, H, I)
+    y = torch.full((T + 3, I), 7.0, dtype=torch.bfloat16, device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        ppas.ppas_gateup_swiglu(x, wp, y, T, H, I, err)
     torch.cuda.synchronize()
     assert int(err.item()) == 0
     assert bool((y[T:] == 7.0).all())
