@@ -27,8 +27,9 @@
 // 5.8 of its 13.3 us, per-CTA timestamps), so the tail is kept short: the
 // ticket is claimed before the merges by a reduction nobody waits for, one
 // thread fences instead of all, the heads of a merge are independent
-// loads, and the last CTA has up to 20 partials in flight.  One row x 25k,
-// 16/2 heads, append + attention: 14.3 -> 13.0 us a layer.  (Claiming at entry
+// loads, and the last CTA merges up to 20 partials in one round, weights in
+// registers.  One row x 25k, 16/2 heads, append + attention: 14.3 -> 12.8 us
+// a layer; 8 rows x 25k 37.4 -> 36.8.  (Claiming at entry
 // cost the page loop 1 %: 96 rows of 17-4100 tokens 270.8 -> 274.5 us.)
 #include <math.h>
 
@@ -441,59 +442,79 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
         }
         if (prev < 0) report_error(p.err, PPAS_DEVERR_TIMEOUT);  // the word was never claimed
         s_last = (prev == n_parts - 1);
-        if (s_last) *ctr = 0;  // also ready for a replay with the same tag (a captured graph)
         __threadfence();
     }
     decode_cta_sync<kPartial>();
     if (!s_last) return;
-    // Warp hh merges head hh on its own (lane: 4 columns).  The first kBatch
-    // splits' O go out before the weights are known, so their latency hides
-    // that of the (m, l) round; the weights w = 2^(m - M) stay in a
-    // shared-memory row of the warp (the rings are free), 1 / L is applied
-    // at the end.
+    if (tid == 0) *ctr = 0;  // ready for a replay with the same tag (a captured graph)
+    // Warp hh merges head hh on its own (lane: 4 columns)
     const int ns = n_parts;
     const int hh = warp, c4 = lane;
     if (hh >= g) return;
     const int head = kvh * g + hh;
     const float4 *po = reinterpret_cast<const float4 *>(p.part_o) + c4;
+    const float2 *pml = reinterpret_cast<const float2 *>(p.part_ml);
     auto part_index = [&](int s_) { return static_cast<int64_t>(row.part_base + s_) * p.n_q_heads + head; };
+    auto warp_max = [](float x) {
+#pragma unroll
+        for (int o_ = 16; o_ >= 1; o_ >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o_));
+        return x;
+    };
+    auto warp_sum = [](float x) {
+#pragma unroll
+        for (int o_ = 16; o_ >= 1; o_ >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o_);
+        return x;
+    };
     constexpr int kBatch = 20;  // a one-row step in clusters has 18 or 19 partials: one round
     float4 ov[kBatch];
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k)
-        ov[k] = k < ns ? __ldcg(po + part_index(k) * (kHeadDim / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float *wm = reinterpret_cast<float *>(sg) + hh * 2 * kMaxDecodeSplitsPerRow;  // [ns] m, then w
-    float *wl = wm + kMaxDecodeSplitsPerRow;                                     // [ns] l
-    float M = -INFINITY;
-    for (int s_ = lane; s_ < ns; s_ += 32) {
-        const float2 ml = __ldcg(reinterpret_cast<const float2 *>(p.part_ml + part_index(s_) * 2));
-        wm[s_] = ml.x;
-        wl[s_] = ml.y;
-        M = fmaxf(M, ml.x);
-    }
-#pragma unroll
-    for (int o_ = 16; o_ >= 1; o_ >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o_));
-    float L = 0.f;
-    for (int s_ = lane; s_ < ns; s_ += 32) {
-        const float m = wm[s_];
-        const float f = m == -INFINITY ? 0.f : ex2(m - M);
-        wm[s_] = f;
-        L += f * wl[s_];
-    }
-#pragma unroll
-    for (int o_ = 16; o_ >= 1; o_ >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o_);
-    __syncwarp();
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < ns; s0 += kBatch) {
-        if (s0 > 0) {
+    float L;
+    auto load_o = [&](int s0) {
 #pragma unroll
-            for (int k = 0; k < kBatch; ++k)
-                ov[k] = s0 + k < ns ? __ldcg(po + part_index(s0 + k) * (kHeadDim / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < kBatch; ++k)
+            ov[k] = s0 + k < ns ? __ldcg(po + part_index(s0 + k) * (kHeadDim / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    auto add_o = [&](int k, float f) {
+        acc = make_float4(acc.x + f * ov[k].x, acc.y + f * ov[k].y, acc.z + f * ov[k].z, acc.w + f * ov[k].w);
+    };
+    if (ns <= kBatch) {
+        // one round: lane s holds split s's (m, l) and weight w = 2^(m - M); its
+        // load goes first, so the weights are there when the O are
+        const float2 ml = lane < ns ? __ldcg(pml + part_index(lane)) : make_float2(-INFINITY, 0.f);
+        load_o(0);
+        const float M = warp_max(ml.x);
+        const float f = ml.x == -INFINITY ? 0.f : ex2(ml.x - M);
+        L = warp_sum(f * ml.y);
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) add_o(k, __shfl_sync(0xffffffffu, f, k));
+    } else {
+        // the first splits' O go out before the weights are known, so their
+        // latency hides that of the (m, l) round; the weights stay in a
+        // shared-memory row of the warp (the rings are free)
+        load_o(0);
+        float *wm = reinterpret_cast<float *>(sg) + hh * 2 * kMaxDecodeSplitsPerRow;  // [ns] m, then w
+        float *wl = wm + kMaxDecodeSplitsPerRow;                                     // [ns] l
+        float M = -INFINITY;
+        for (int s_ = lane; s_ < ns; s_ += 32) {
+            const float2 ml = __ldcg(pml + part_index(s_));
+            wm[s_] = ml.x;
+            wl[s_] = ml.y;
+            M = fmaxf(M, ml.x);
         }
+        M = warp_max(M);
+        L = 0.f;
+        for (int s_ = lane; s_ < ns; s_ += 32) {
+            const float m = wm[s_];
+            const float f = m == -INFINITY ? 0.f : ex2(m - M);
+            wm[s_] = f;
+            L += f * wl[s_];
+        }
+        L = warp_sum(L);
+        __syncwarp();
+        for (int s0 = 0; s0 < ns; s0 += kBatch) {
+            if (s0 > 0) load_o(s0);
 #pragma unroll
-        for (int k = 0; k < kBatch; ++k) {
-            const float f = s0 + k < ns ? wm[s0 + k] : 0.f;
-            acc = make_float4(acc.x + f * ov[k].x, acc.y + f * ov[k].y, acc.z + f * ov[k].z, acc.w + f * ov[k].w);
+            for (int k = 0; k < kBatch; ++k) add_o(k, s0 + k < ns ? wm[s0 + k] : 0.f);
         }
     }
     const float inv_l = 1.f / L;
