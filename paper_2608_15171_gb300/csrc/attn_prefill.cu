@@ -754,66 +754,83 @@ static_assert(kDecodeThreads == 8 * 32 && kDecodeSmemBytes <= kSmemBytes,
 // Combines the pieces of a split unit:
 //   o = sum_i 2^(m_i - M) o_i / sum_i 2^(m_i - M) l_i,  M = max_i m_i
 // (m in log2 units), taking the pieces four at a time with the running
-// maximum (exact up to rounding).  One thread per (query row, 4 columns):
-// CTA (unit, head t, chunk c4, quarter) covers 32 rows x 32 columns; a warp
-// reads eight runs of 64 bytes of a partial.
+// maximum (exact up to rounding).  CTA (unit, head t, 32 rows, 64 columns); a
+// warp takes the 32 rows (a lane a row) and 8 columns, so a load of a partial
+// is 512 contiguous bytes, a lane has up to 12 loads in flight, and a bf16
+// store is 16 bytes.  Bound by the latency of its rounds of four pieces and by
+// L2.  With one float4 a thread and four rows a warp it took 5.2 us of a
+// 512-token layer's 19.6 and 7.7 of the 4 x 512 step's 137; the layers now take
+// 18.5-18.8 and 134 (16 columns a lane: 18.7 and 135.4; 4: 18.6 and 135.6;
+// eight pieces a round: 19.6 and 136.8), 128 tokens over 25,000 (19 pieces a
+// unit) 28.3 -> 25.6.
 __global__ void __launch_bounds__(256) prefill_merge_kernel(const __grid_constant__ MergeParams p) {
     grid_dep_wait();  // the partials come from the prefill launch before this one
     const int hpc = p.heads_per_cta;
-    const int lin = (blockIdx.x & 3) * 256 + threadIdx.x;  // 0..1023 within (unit, head, chunk)
-    const int r = lin >> 3, j4 = lin & 7;
-    int rest = blockIdx.x >> 2;
-    const int c4 = rest & 3;
-    rest >>= 2;
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) + 8 * (blockIdx.x & 1);
+    const int r = ((blockIdx.x >> 1) & 3) * 32 + lane;
+    int rest = blockIdx.x >> 3;
     const int t = rest % hpc;
     const MergeUnit mu = p.units[rest / hpc];
     const int ns = mu.n_splits;
-    auto pblk = [&](int i) { return (static_cast<int64_t>(mu.part) + i) * hpc + t; };
+    constexpr int kC = 2;  // 16-byte chunks of a lane
     float M = -INFINITY, L = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 acc[kC];
+#pragma unroll
+    for (int c = 0; c < kC; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i0 = 0; i0 < ns; i0 += 4) {
         float2 ml[4];
-        float4 o[4];
+        float4 o[4][kC];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (i0 + k < ns) {
-                const int64_t b = pblk(i0 + k);
-                ml[k] = __ldcg(reinterpret_cast<const float2 *>(p.part_ml + (b * kTileQ + r) * 2));
-                o[k] = __ldcg(reinterpret_cast<const float4 *>(p.part_o) + (b * (kHeadDim / 4) + c4 * 8 + j4) * kTileQ + r);
-            } else {
-                ml[k] = make_float2(-INFINITY, 0.f);
-                o[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+            const int64_t b = (static_cast<int64_t>(mu.part) + i0 + k) * hpc + t;
+            ml[k] = i0 + k < ns ? __ldcg(reinterpret_cast<const float2 *>(p.part_ml + (b * kTileQ + r) * 2))
+                                : make_float2(-INFINITY, 0.f);
+#pragma unroll
+            for (int c = 0; c < kC; ++c)
+                o[k][c] = i0 + k < ns ? __ldcg(reinterpret_cast<const float4 *>(p.part_o) +
+                                               (b * (kHeadDim / 4) + warp * kC + c) * kTileQ + r)
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         const float mn = fmaxf(fmaxf(M, fmaxf(ml[0].x, ml[1].x)), fmaxf(ml[2].x, ml[3].x));
         if (mn == -INFINITY) continue;  // every key of these pieces is masked for this row
         const float sc = M == -INFINITY ? 0.f : ex2(M - mn);
         L *= sc;
-        acc = make_float4(acc.x * sc, acc.y * sc, acc.z * sc, acc.w * sc);
+#pragma unroll
+        for (int c = 0; c < kC; ++c) acc[c] = make_float4(acc[c].x * sc, acc[c].y * sc, acc[c].z * sc, acc[c].w * sc);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const float f = ml[k].x == -INFINITY ? 0.f : ex2(ml[k].x - mn);
             L += f * ml[k].y;
-            acc = make_float4(acc.x + f * o[k].x, acc.y + f * o[k].y, acc.z + f * o[k].z, acc.w + f * o[k].w);
+#pragma unroll
+            for (int c = 0; c < kC; ++c)
+                acc[c] = make_float4(acc[c].x + f * o[k][c].x, acc[c].y + f * o[k][c].y, acc[c].z + f * o[k][c].z,
+                                     acc[c].w + f * o[k][c].w);
         }
         M = mn;
     }
     if (r >= mu.rows_valid) return;
     const float inv_l = 1.f / L;
     const int64_t orow = static_cast<int64_t>(mu.out_row0 + r) * p.n_q_heads + mu.head0 + t;
-    const int64_t col = orow * kHeadDim + c4 * 32 + j4 * 4;
+    const int64_t col = orow * kHeadDim + warp * (4 * kC);
     if (p.out_fp32) {
-        *reinterpret_cast<float4 *>(static_cast<float *>(p.out) + col) =
-            make_float4(acc.x * inv_l, acc.y * inv_l, acc.z * inv_l, acc.w * inv_l);
+        float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(p.out) + col);
+#pragma unroll
+        for (int c = 0; c < kC; ++c)
+            dst[c] = make_float4(acc[c].x * inv_l, acc[c].y * inv_l, acc[c].z * inv_l, acc[c].w * inv_l);
     } else {
-        *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(p.out) + col) =
-            make_uint2(pack_bf16x2(acc.x * inv_l, acc.y * inv_l), pack_bf16x2(acc.z * inv_l, acc.w * inv_l));
+        uint4 *dst = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p.out) + col);
+#pragma unroll
+        for (int c = 0; c < kC; c += 2)
+            dst[c / 2] = make_uint4(pack_bf16x2(acc[c].x * inv_l, acc[c].y * inv_l),
+                                    pack_bf16x2(acc[c].z * inv_l, acc[c].w * inv_l),
+                                    pack_bf16x2(acc[c + 1].x * inv_l, acc[c + 1].y * inv_l),
+                                    pack_bf16x2(acc[c + 1].z * inv_l, acc[c + 1].w * inv_l));
     }
 }
 
 cudaError_t launch_prefill_merge(const MergeParams &p, cudaStream_t st) {
     if (p.n_units <= 0) return cudaSuccess;
-    PdlLaunch l(dim3(p.n_units * p.heads_per_cta * 16), dim3(256), 0, st);
+    PdlLaunch l(dim3(p.n_units * p.heads_per_cta * 8), dim3(256), 0, st);
     return cudaLaunchKernelEx(&l.cfg, prefill_merge_kernel, p);
 }
 
