@@ -10,10 +10,15 @@
 // swizzle) into a 3-stage ring per warp (eight warps, so eight threads issue
 // copies; one issuing thread alone moves only ~7 B/clk); the split's page ids
 // are staged in shared memory first.  Each warp computes
-//   S^T[heads x 16 keys] = Q[heads x 128] . K_page^T     (mma.sync m16n8k16)
+//   S^T[16 keys x heads] = K_page[16 x 128] . Q^T        (mma.sync m16n8k16)
 //   online softmax per head (fp32, exp2 domain)
-//   O[heads x 128] += P[heads x 16 keys] . V_page         (mma.sync m16n8k16)
-// with the group's q-heads as the MMA rows (rows >= group are zero).  The
+//   O^T[128 x heads] += V_page^T[128 x 16 keys] . P^T     (mma.sync m16n8k16)
+// with the group's q-heads as the MMA's 8 columns (columns >= group are zero):
+// 16 MMAs a page.  With the heads as its 16 rows, half of them always empty, a
+// page took 48, and a step bound by one SM's rate (few rows, or decode rows
+// beside prefill items) waited for them: 1 row x 25k (16/2 heads) 13.0 -> 12.6
+// us a layer, 8 rows 36.8 -> 36.1, 16 rows x 30k (32/8) 283.5 -> 281.3, 4 x 512
+// with 8 decodes 134.5 -> 131.5.  The
 // warps merge their (m, l, O) in shared memory; with several splits the
 // partial goes to the workspace and the last CTA of the (row, kv-head) to
 // finish merges all splits:
@@ -29,8 +34,8 @@
 // thread fences instead of all, the heads of a merge are independent
 // loads, and the last CTA merges up to 20 partials in one round, weights in
 // registers.  One row x 25k, 16/2 heads, append + attention: 14.3 -> 12.8 us
-// a layer; 8 rows x 25k 37.4 -> 36.8.  (Claiming at entry
-// cost the page loop 1 %: 96 rows of 17-4100 tokens 270.8 -> 274.5 us.)
+// a layer; 8 rows x 25k 37.4 -> 36.8.  (Claiming at entry the page
+// loop 1 %: 96 rows of 17-4100 tokens 270.8 -> 274.5 us.)
 #include <math.h>
 
 #include "ppas_device.cuh"
@@ -56,7 +61,10 @@ constexpr uint32_t kSmemBytes = kOffClusterRecv + kClusterRecvBytes + 1024;
 static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 // merge scratch (aliases the rings once every warp is done)
 constexpr int kMaxGroup = 8;
-static_assert(kDecodeWarps * kMaxGroup * (2 + kHeadDim) * 4 <= static_cast<int>(kOffBar), "merge scratch");
+// a warp's O rows in the merge scratch: four floats apart from 128, so that
+// the accumulators' columns fall into different banks
+constexpr int kCoStride = kHeadDim + 4;
+static_assert(kDecodeWarps * kMaxGroup * (2 + kCoStride) * 4 <= static_cast<int>(kOffBar), "merge scratch");
 static_assert(2 * kMaxDecodeSplitsPerRow * kMaxGroup * 4 <= static_cast<int>(kOffBar), "split weights");
 static_assert(kDecodeWarps >= kMaxGroup, "the split merge gives each head of a group one warp");
 static_assert(kClusterRecvBytes == kMaxCluster * kMaxGroup * (kHeadDim + 2) * 4, "cluster slots");
@@ -77,6 +85,13 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a
         "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// transposes an 8 x 8 matrix of 16-bit values held one row to four lanes
+__device__ __forceinline__ uint32_t movmatrix_t(uint32_t a) {
+    uint32_t d;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+    return d;
 }
 
 // byte offset of 16-byte chunk `chunk` (0..15 over 128 columns) of `row` in
@@ -182,26 +197,26 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
     };
     for (int i = 0; i < min(kDecodeStages, my_count); ++i) issue(i);
 
-    // ---- Q as the A operand: rows = the group's heads, k = head dims
+    // ---- Q as the B operand: n = the group's heads, k = head dims
     const int hr = lane >> 2, c = lane & 3;
-    uint32_t qa[8][4];
+    uint32_t qb[8][2];
     {
         const bool valid = hr < g;
         const uint32_t *qrow = reinterpret_cast<const uint32_t *>(
             p.q + (static_cast<int64_t>(row.q_row) * p.n_q_heads + kvh * g + (valid ? hr : 0)) * kHeadDim);
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
-            qa[kk][0] = valid ? __ldg(qrow + kk * 8 + c) : 0u;
-            qa[kk][1] = 0u;
-            qa[kk][2] = valid ? __ldg(qrow + kk * 8 + 4 + c) : 0u;
-            qa[kk][3] = 0u;
+            qb[kk][0] = valid ? __ldg(qrow + kk * 8 + c) : 0u;
+            qb[kk][1] = valid ? __ldg(qrow + kk * 8 + 4 + c) : 0u;
         }
     }
 
-    float m_run = -INFINITY, l_run = 0.f;
-    float o[16][4];
+    // accumulators: this lane has tokens hr and hr + 8 of a page's S, head
+    // dims 16 n + hr and 16 n + hr + 8 of O, and heads 2c, 2c + 1 of both
+    float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;  // l: over this lane's tokens
+    float o[8][4];
 #pragma unroll
-    for (int n = 0; n < 16; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
+    for (int n = 0; n < 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
     const float sl2 = p.scale_log2;
     int consumed = 0;
 
@@ -227,47 +242,49 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
             fence_proxy_async_smem();
             __syncwarp();
         }
-        // S = Q K^T for the 16 tokens of the page (two n-tiles of 8 tokens)
-        float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
-        {
-            const int mi = lane >> 3, ri = lane & 7;
-            const int tok = (mi >> 1) * 8 + ri;
+        // S^T = K Q^T: 16 tokens x 8 heads, k over the head dims (two chains)
+        float sa[4] = {0.f, 0.f, 0.f, 0.f}, sc[4] = {0.f, 0.f, 0.f, 0.f};
+        const int mi = lane >> 3, ri = lane & 7;
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-                uint32_t b0, b1, b2, b3;
-                ldsm_x4(kb + swz(tok, kk * 2 + (mi & 1)), b0, b1, b2, b3);
-                mma_bf16_16816(s0, qa[kk], b0, b1);
-                mma_bf16_16816(s1, qa[kk], b2, b3);
-            }
+        for (int kk = 0; kk < 8; kk += 2) {
+            uint32_t a[4];
+            ldsm_x4(kb + swz((mi & 1) * 8 + ri, kk * 2 + (mi >> 1)), a[0], a[1], a[2], a[3]);
+            mma_bf16_16816(sa, a, qb[kk][0], qb[kk][1]);
+            ldsm_x4(kb + swz((mi & 1) * 8 + ri, kk * 2 + 2 + (mi >> 1)), a[0], a[1], a[2], a[3]);
+            mma_bf16_16816(sc, a, qb[kk + 1][0], qb[kk + 1][1]);
         }
-        const float x0 = (2 * c < valid) ? s0[0] * sl2 : -INFINITY;
-        const float x1 = (2 * c + 1 < valid) ? s0[1] * sl2 : -INFINITY;
-        const float x2 = (8 + 2 * c < valid) ? s1[0] * sl2 : -INFINITY;
-        const float x3 = (9 + 2 * c < valid) ? s1[1] * sl2 : -INFINITY;
-        float mx = fmaxf(fmaxf(x0, x1), fmaxf(x2, x3));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(m_run, mx);
-        const float alpha = ex2(m_run - m_new);
-        m_run = m_new;
-        const float e0 = ex2(x0 - m_new), e1 = ex2(x1 - m_new), e2 = ex2(x2 - m_new), e3 = ex2(x3 - m_new);
-        l_run = l_run * alpha + (e0 + e1) + (e2 + e3);
+        const float x0 = hr < valid ? (sa[0] + sc[0]) * sl2 : -INFINITY;  // (token hr, head 2c)
+        const float x1 = hr < valid ? (sa[1] + sc[1]) * sl2 : -INFINITY;
+        const float x2 = hr + 8 < valid ? (sa[2] + sc[2]) * sl2 : -INFINITY;  // (token hr + 8, head 2c)
+        const float x3 = hr + 8 < valid ? (sa[3] + sc[3]) * sl2 : -INFINITY;
+        float mx0 = fmaxf(x0, x2), mx1 = fmaxf(x1, x3);
 #pragma unroll
-        for (int n = 0; n < 16; ++n) {
-            o[n][0] *= alpha;
-            o[n][1] *= alpha;
+        for (int o_ = 4; o_ <= 16; o_ <<= 1) {
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o_));
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o_));
         }
-        const uint32_t pa[4] = {pack_bf16x2(e0, e1), 0u, pack_bf16x2(e2, e3), 0u};
-        {
-            const int mi = lane >> 3, ri = lane & 7;
-            const int tok = (mi & 1) * 8 + ri;
+        mx0 = fmaxf(m0, mx0);
+        mx1 = fmaxf(m1, mx1);
+        const float al0 = ex2(m0 - mx0), al1 = ex2(m1 - mx1);
+        m0 = mx0;
+        m1 = mx1;
+        const float e0 = ex2(x0 - m0), e1 = ex2(x1 - m1), e2 = ex2(x2 - m0), e3 = ex2(x3 - m1);
+        l0 = l0 * al0 + (e0 + e2);
+        l1 = l1 * al1 + (e1 + e3);
 #pragma unroll
-            for (int n2 = 0; n2 < 8; ++n2) {
-                uint32_t b0, b1, b2, b3;
-                ldsm_x4_t(vb + swz(tok, n2 * 2 + (mi >> 1)), b0, b1, b2, b3);
-                mma_bf16_16816(o[2 * n2], pa, b0, b1);
-                mma_bf16_16816(o[2 * n2 + 1], pa, b2, b3);
-            }
+        for (int n = 0; n < 8; ++n) {
+            o[n][0] *= al0;
+            o[n][1] *= al1;
+            o[n][2] *= al0;
+            o[n][3] *= al1;
+        }
+        // O^T += V^T P^T: 16 head dims x 8 heads at a time, k over the tokens
+        const uint32_t p0 = movmatrix_t(pack_bf16x2(e0, e1)), p1 = movmatrix_t(pack_bf16x2(e2, e3));
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            uint32_t a[4];
+            ldsm_x4_t(vb + swz((mi >> 1) * 8 + ri, n * 2 + (mi & 1)), a[0], a[1], a[2], a[3]);
+            mma_bf16_16816(o[n], a, p0, p1);
         }
         __syncwarp();
         if (i + kDecodeStages < my_count) issue(i + kDecodeStages);
@@ -292,21 +309,32 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
     const unsigned long long ticket0 = p.launch_tag << 16;
     if (tid == 0 && row.n_splits > 1 && crank == 0) atomicMax(ctr, ticket0);
 
-    l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
-    l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+#pragma unroll
+    for (int o_ = 4; o_ <= 16; o_ <<= 1) {
+        l0 += __shfl_xor_sync(0xffffffffu, l0, o_);
+        l1 += __shfl_xor_sync(0xffffffffu, l1, o_);
+    }
 
     decode_cta_sync<kPartial>();  // rings are free from here on
     float *cm = reinterpret_cast<float *>(sg);
     float *cl = cm + kDecodeWarps * kMaxGroup;
     float *co = cl + kDecodeWarps * kMaxGroup;
-    if (hr < g) {
-        if (c == 0) {
-            cm[warp * kMaxGroup + hr] = m_run;
-            cl[warp * kMaxGroup + hr] = l_run;
-        }
-        float *dst = co + (warp * kMaxGroup + hr) * kHeadDim;
+    // this lane's heads 2c, 2c + 1 (those past the group are left out)
 #pragma unroll
-        for (int n = 0; n < 16; ++n) *reinterpret_cast<float2 *>(dst + n * 8 + 2 * c) = make_float2(o[n][0], o[n][1]);
+    for (int x = 0; x < 2; ++x) {
+        const int hh = 2 * c + x;
+        if (hh < g) {
+            if (hr == 0) {
+                cm[warp * kMaxGroup + hh] = x ? m1 : m0;
+                cl[warp * kMaxGroup + hh] = x ? l1 : l0;
+            }
+            float *dst = co + (warp * kMaxGroup + hh) * kCoStride + hr;
+#pragma unroll
+            for (int n = 0; n < 8; ++n) {
+                dst[16 * n] = o[n][x];
+                dst[16 * n + 8] = o[n][2 + x];
+            }
+        }
     }
     decode_cta_sync<kPartial>();
     // (in a cluster an aborted CTA carries on to the cluster barrier below)
@@ -343,7 +371,7 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
             // cluster plan may hold) has m = -inf and weight 0
             const float f = m[w] == -INFINITY ? 0.f : ex2(m[w] - Mh[i]);
             Lh[i] += f * cl[w * kMaxGroup + hh];
-            Oh[i] += f * co[(w * kMaxGroup + hh) * kHeadDim + t];
+            Oh[i] += f * co[(w * kMaxGroup + hh) * kCoStride + t];
         }
     }
 #pragma unroll
