@@ -34,8 +34,8 @@
 // thread fences instead of all, the heads of a merge are independent
 // loads, and the last CTA merges up to 20 partials in one round, weights in
 // registers.  One row x 25k, 16/2 heads, append + attention: 14.3 -> 12.8 us
-// a layer; 8 rows x 25k 37.4 -> 36.8.  (Claiming at entry the page
-// loop 1 %: 96 rows of 17-4100 tokens 270.8 -> 274.5 us.)
+// a layer; 8 rows x 25k 37.4 -> 36.8.  (Claiming at entry cost
+// the page loop 1 %: 96 rows of 17-4100 tokens 270.8 -> 274.5 us.)
 #include <math.h>
 
 #include "ppas_device.cuh"

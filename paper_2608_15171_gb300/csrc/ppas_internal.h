@@ -156,6 +156,7 @@ constexpr int kMaxDecodeSplitsPerRow = 2048;   // the merge keeps every split's 
 constexpr int64_t kMaxDecodeCtx = int64_t{kMaxDecodeSplitsPerRow} * kDecodeMaxPagesPerSplit * 16;
 constexpr int kMaxDecodeRows = 256;
 constexpr int kDecodeMinPagesPerSplit = 16;
+constexpr int kDecodeMinPagesToHalve = 128;  // splits of a mixed step's last rows that may be halved
 
 struct DecodeRow {
     int32_t q_row;       // row of packed q / out
@@ -248,9 +249,11 @@ DecodeClusterCaps decode_cluster_caps();  // the current device's, cached
 
 // decode splits for a device of num_sms SMs: one wave of CTAs where the
 // split-size limits allow it.  A step of decode rows only may run its
-// splits in clusters (caps: what the device holds co-resident).
+// splits in clusters (caps: what the device holds co-resident).  fine_tail:
+// the last rows of a step that has prefill rows too get shorter splits.
 DecodePlan plan_decode(int32_t n_seqs, const int32_t *q_lens, const int32_t *ctx_lens, int32_t n_q_heads,
-                       int32_t n_kv_heads, int32_t num_sms, const DecodeClusterCaps &caps = {});
+                       int32_t n_kv_heads, int32_t num_sms, const DecodeClusterCaps &caps = {},
+                       bool fine_tail = false);
 
 int32_t device_sm_count();
 // SMs the current device's step plans are made for: its SM count, at most
