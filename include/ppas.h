@@ -260,6 +260,8 @@ ppas_status ppas_attention_step(const void *q, const void *k_cache, const void *
  * PPAS_ERR_UNSUPPORTED; pointers 16-byte aligned, else PPAS_ERR_INVALID_ARG;
  * n_tokens == 0 is a no-op.  d_err_flag (device int32 or NULL) records
  * PPAS_DEVERR_TIMEOUT if a bounded wait runs out.
+ * ppas_gateup_swiglu is one launch, with programmatic stream serialization as
+ * the attention kernels (its set-up may overlap the kernel before it).
  * ------------------------------------------------------------------------- */
 ppas_status ppas_gateup_pack(const void *w, void *w_packed, int32_t hidden, int32_t inter, void *stream);
 ppas_status ppas_gateup_swiglu(const void *x, const void *w_packed, void *y, int32_t n_tokens, int32_t hidden,
