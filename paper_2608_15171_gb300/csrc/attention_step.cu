@@ -491,7 +491,13 @@ PrefillPlan plan_prefill(int32_t n_seqs, const int32_t *q_lens, const int32_t *c
                     per_cta[c].push_back(pc.second);
                 }
             const int64_t cut_span = span(filled);
-            if (lp.n_part == 0 || (!needs_cut && cut_span + kPrefillMergeCost >= whole_span)) {
+            // the partials and the merge cost kPrefillMergeCost tiles, two more in
+            // a step of 64 tiles a CTA or longer, where many CTAs write them at
+            // once (2048 tokens, longest CTA 19 tiles against 14 cut: 26.1 us a
+            // layer whole, 25.0 cut; 16384 tokens, 464 against about 458: 640 whole,
+            // 655 cut)
+            const int64_t cost = kPrefillMergeCost + std::min<int64_t>(2, whole_span / 32);
+            if (lp.n_part == 0 || (!needs_cut && cut_span + cost >= whole_span)) {
                 per_cta = std::move(whole);  // not worth the partials
                 lp.split_units.clear();
                 lp.n_part = 0;

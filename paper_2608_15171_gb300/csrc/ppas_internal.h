@@ -43,7 +43,7 @@ constexpr int kPrefillMinPiece = 4;     // shortest piece of a split unit, in KV
 // TMEM loses ~7e-7 of |O| per tile, so pieces are capped and the merge
 // (ordinary fp32) combines them
 constexpr int kPrefillMaxPiece = 512;
-constexpr int kPrefillMergeCost = 6;    // partial writes and the merge launch, in KV tiles
+constexpr int kPrefillMergeCost = 4;    // partial writes and the merge launch, in KV tiles
 constexpr uint16_t kNoPart = 0xFFFF;    // an item of an unsplit unit
 
 struct PrefillSeq {
