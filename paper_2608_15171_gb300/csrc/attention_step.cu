@@ -1008,15 +1008,17 @@ extern "C" ppas_status ppas_gateup_swiglu(const void *x, const void *w_packed, v
     gp.inter = inter;
     gp.err = d_err_flag;
     const bool few = n_tokens <= kFewTokens;
+    const int sms = device_sm_count();
     CUtensorMap tm_x, tm_w;
     if (!encode_bf16_2d(&tm_x, x, static_cast<uint64_t>(hidden), static_cast<uint64_t>(n_tokens), 64,
                         few ? static_cast<uint32_t>((n_tokens + 15) & ~15) : 128) ||
         !encode_bf16_2d(&tm_w, w_packed, static_cast<uint64_t>(hidden), 2ull * inter, 64, few ? 64 : 128))
         return PPAS_ERR_CUDA;
     if (few)
-        return launch_gateup_few(tm_x, tm_w, gp, static_cast<cudaStream_t>(stream)) == cudaSuccess ? PPAS_OK
-                                                                                                   : PPAS_ERR_CUDA;
-    const GateUpPlan gu = plan_gateup(n_tokens, inter, std::max(1, device_sm_count() / 2));
+        return launch_gateup_few(tm_x, tm_w, gp, sms, static_cast<cudaStream_t>(stream)) == cudaSuccess
+                   ? PPAS_OK
+                   : PPAS_ERR_CUDA;
+    const GateUpPlan gu = plan_gateup(n_tokens, inter, std::max(1, sms / 2));
     gp.n_full = gu.n_full;
     gp.cut = gu.cut;
     gp.n_items = gu.n_items;

@@ -313,17 +313,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
 constexpr int kFF = 64;  // features per CTA
 constexpr uint32_t kFewA = 128 * kGK * 2;  // weight tile of a K block: 16 KB
 constexpr uint32_t kFewRing = 112640;      // ring bytes at most: two CTAs share an SM
-constexpr int kFewMaxStages = 6;
+constexpr uint32_t kFewRingAlone = 225280; // and where no SM gets a second CTA
+constexpr int kFewMaxStages = 12;
 
 // accumulator columns to allocate: a power of two, at least 32
 __host__ __device__ constexpr int few_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : 128; }
 __host__ __device__ constexpr uint32_t few_stage(int n) { return kFewA + static_cast<uint32_t>(n) * kGK * 2; }
-__host__ __device__ constexpr int few_stages(int n) {
-    return static_cast<int>(kFewRing / few_stage(n)) < kFewMaxStages ? static_cast<int>(kFewRing / few_stage(n))
-                                                                     : kFewMaxStages;
+__host__ __device__ constexpr int few_stages(int n, uint32_t ring) {
+    return static_cast<int>(ring / few_stage(n)) < kFewMaxStages ? static_cast<int>(ring / few_stage(n))
+                                                                 : kFewMaxStages;
 }
-static_assert(few_stages(kFewTokens) >= 3, "ring depth");
-static_assert(kFewTokens * 128 * 4 <= few_stages(kFewTokens) * few_stage(kFewTokens), "epilogue buffer in the ring");
+static_assert(few_stages(kFewTokens, kFewRing) >= 3, "ring depth");
+static_assert(kFewTokens * 128 * 4 <= few_stages(kFewTokens, kFewRing) * few_stage(kFewTokens),
+              "epilogue buffer in the ring");
 
 __global__ void __launch_bounds__(kGThreads, 2)
     gateup_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
@@ -344,7 +346,8 @@ __global__ void __launch_bounds__(kGThreads, 2)
 
     const int n = (p.n_tokens + 15) & ~15;
     const uint32_t stage = few_stage(n);
-    const int stages = few_stages(n);
+    // (computed: as a parameter of the launch, calls of 5 us took 0.1 more)
+    const int stages = few_stages(n, p.alone ? kFewRingAlone : kFewRing);
     const int k_blocks = p.hidden / kGK;
     const int f0 = blockIdx.x * kFF;                       // first feature
     const int w_row = (f0 / 128) * 256 + (f0 % 128);       // its gate row in the packed weight; up: + 128
@@ -353,16 +356,16 @@ __global__ void __launch_bounds__(kGThreads, 2)
         tmem_alloc(smem_u32(&tmem_base), few_cols(n));
         tmem_relinquish();
     }
-    if (tid == 0) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(full(s), 1);
-            mbar_init(empty(s), 1);
+    if (tid < stages) {
+        mbar_init(full(tid), 1);
+        mbar_init(empty(tid), 1);
+        if (tid == 0) {
+            mbar_init(done, 1);
+            *abort_flag = 0;
+            prefetch_tmap(&tm_x);
+            prefetch_tmap(&tm_w);
         }
-        mbar_init(done, 1);
-        *abort_flag = 0;
         fence_mbar_init();
-        prefetch_tmap(&tm_x);
-        prefetch_tmap(&tm_w);
     }
     tc_fence_before();
     __syncthreads();
@@ -486,15 +489,26 @@ cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, cons
 // 128 tokens every CTA would read more of x than of the weights, and the
 // ring would fall below three stages: those calls take the kernel above (129
 // tokens: 24.2).
-cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p,
+//
+// With no more CTAs than SMs (inter <= 9728) each has an SM to itself: fewer SMs
+// stream, so each has to keep more bytes in flight, and gets the longer ring.
+// Times with kFewRing and with kFewRingAlone: hidden 4096, inter 4096 (67 MB,
+// 64 CTAs): 24 tokens 16.8 -> 14.1 us, 64: 20.6 -> 14.8, 128: 24.8 -> 17.9 (the
+// kernel above: 19.0, 19.2, 19.8); hidden 2048, inter 5632: 24 tokens 11.5 ->
+// 10.7, 128: 16.0 -> 12.7; hidden 1024, inter 2816: 128 tokens 6.7 -> 6.1, 24
+// tokens 4.9 and 4.9.
+cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p, int sms,
                               cudaStream_t st) {
     static std::atomic<uint64_t> smem_set{0};
     const cudaError_t e =
-        ensure_smem_limit(gateup_few_kernel, static_cast<int>(kFewRing + 1024), smem_set);
+        ensure_smem_limit(gateup_few_kernel, static_cast<int>(kFewRingAlone + 1024), smem_set);
     if (e != cudaSuccess) return e;
     const int n = (p.n_tokens + 15) & ~15;
-    PdlLaunch l(dim3(p.inter / kFF), dim3(kGThreads), few_stages(n) * few_stage(n) + 1024, st);
-    return cudaLaunchKernelEx(&l.cfg, gateup_few_kernel, tm_x, tm_w, p);
+    GateUpParams fp = p;
+    fp.alone = p.inter / kFF <= sms;
+    const int stages = few_stages(n, fp.alone ? kFewRingAlone : kFewRing);
+    PdlLaunch l(dim3(p.inter / kFF), dim3(kGThreads), stages * few_stage(n) + 1024, st);
+    return cudaLaunchKernelEx(&l.cfg, gateup_few_kernel, tm_x, tm_w, fp);
 }
 
 cudaError_t launch_gateup_pack(const void *w, void *wp, int hidden, int inter, cudaStream_t st) {

@@ -272,6 +272,8 @@ struct GateUpParams {
     // (256 tokens x 128 features), the rest slices of 128 / cut features of the
     // tiles after them
     int32_t n_full, cut, n_items;
+    // a launch for few tokens: its CTAs have an SM each (the long ring)
+    int32_t alone;
 };
 struct GateUpPlan {
     int32_t pairs, n_full, cut, n_items;
@@ -291,7 +293,7 @@ cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, cons
 // calls of at most this many tokens take the weight-streaming kernel
 constexpr int kFewTokens = 128;
 // tm_x: box of (n_tokens rounded up to 16) rows; tm_w: box of 64 rows
-cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p,
+cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p, int sms,
                               cudaStream_t st);
 cudaError_t launch_gateup_pack(const void *w, void *wp, int hidden, int inter, cudaStream_t st);
 

@@ -31,6 +31,21 @@ def test_every_element_and_nothing_past_the_tokens(ppas, T, H, I):  # noqa: F811
 
 
 @pytest.mark.parametrize("T,H,I", [
+    (1, 64 * 11, 128),      # the long ring (12 stages), one K block short of it
+    (1, 64 * 12, 256),      # just its length
+    (1, 64 * 25, 128),      # twice, and one
+    (128, 64 * 6, 384),     # the long ring of 6 stages
+    (128, 64 * 7, 384),
+    (50, 64 * 20, 9728),    # a CTA for each of 152 SMs: the long ring
+    (50, 64 * 20, 9856),    # two CTAs more: the short one
+])
+def test_ring_lengths(ppas, T, H, I):  # noqa: F811
+    """K around the length of the long ring, and both sides of the CTA count
+    where the short one takes over."""
+    test_every_element_and_nothing_past_the_tokens(ppas, T, H, I)
+
+
+@pytest.mark.parametrize("T,H,I", [
     (129, 64, 128 * 40),    # 40 tiles: one round of whole tiles
     (200, 128, 128 * 30),   # 30 tiles: halves
     (256, 64, 128 * 19),    # 19 tiles: quarters
