@@ -558,7 +558,7 @@ int32_t decode_reserve_sms(int32_t n_seqs, const int32_t *q_lens, const int32_t 
 
 // Tiles of 256 tokens x 128 features, one at a time to a CTA pair.  The tiles of
 // a last round that would leave at least half the pairs idle are cut into 2 or
-// 4 slices of the features, when those fit one round: 86 tiles (129-256 tokens,
+// 4 slices of the features, when those fit one round: 86 tiles (161-256 tokens,
 // inter 11008) over 76 pairs 28.7 -> 25.0 us, 774 (2056 tokens) 113.1 -> 108.8.
 // A slice takes more than its share (every slice reads the tile's tokens), so
 // slices over several rounds lose: 344 tiles (800 tokens), the last 40 as 160

@@ -317,7 +317,7 @@ constexpr uint32_t kFewRingAlone = 225280; // and where no SM gets a second CTA
 constexpr int kFewMaxStages = 12;
 
 // accumulator columns to allocate: a power of two, at least 32
-__host__ __device__ constexpr int few_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : 128; }
+__host__ __device__ constexpr int few_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : 256; }
 __host__ __device__ constexpr uint32_t few_stage(int n) { return kFewA + static_cast<uint32_t>(n) * kGK * 2; }
 __host__ __device__ constexpr int few_stages(int n, uint32_t ring) {
     return static_cast<int>(ring / few_stage(n)) < kFewMaxStages ? static_cast<int>(ring / few_stage(n))
@@ -485,10 +485,11 @@ cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, cons
 // Times on one GB300, with 128-token tiles before and now (hidden 2048,
 // inter 11008, 90 MB of weights): 1 token 26.5 -> 18.1 us, 8: 25.3 -> 17.8,
 // 32: 22.3 -> 16.9, 64: 22.7 -> 18.6, 128: 23.4 -> 20.5 (the copy bandwidth
-// takes 13.4); hidden 4096, inter 14336 (235 MB), 4 tokens: 55.1 -> 37.7.  Past
-// 128 tokens every CTA would read more of x than of the weights, and the
-// ring would fall below three stages: those calls take the kernel above (129
-// tokens: 24.2).
+// takes 13.4); hidden 4096, inter 14336 (235 MB), 4 tokens: 55.1 -> 37.7.  Against
+// the kernel above: 129 tokens 24.1 there, 20.4 here, 160 tokens 24.2 and 21.1
+// (inter 14336: 45.9 and 43.8; hidden 8192, inter 28672: 157 on both).  Past
+// 160 the ring falls below three stages and the epilogue's buffer outgrows it:
+// those calls take the kernel above.
 //
 // With no more CTAs than SMs (inter <= 9728) each has an SM to itself: fewer SMs
 // stream, so each has to keep more bytes in flight, and gets the longer ring.

@@ -291,7 +291,7 @@ bool encode_bf16_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t
 cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const CUtensorMap &tm_cut,
                           const GateUpParams &p, int pairs, cudaStream_t st);
 // calls of at most this many tokens take the weight-streaming kernel
-constexpr int kFewTokens = 128;
+constexpr int kFewTokens = 160;
 // tm_x: box of (n_tokens rounded up to 16) rows; tm_w: box of 64 rows
 cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p, int sms,
                               cudaStream_t st);

@@ -1,5 +1,5 @@
 """The gate-up kernels at the edges of their ranges.  The weight-streaming one
-(calls of at most 128 tokens): one token, around each multiple of 16 that changes the
+(calls of at most 160 tokens): one token, around each multiple of 16 that changes the
 MMA's N, the largest call it takes and the first one past it; the smallest
 K and feature counts, and K longer than the ring.  Every element against the
 float64 oracle, and the rows after the last token untouched.  The CTA-pair
@@ -14,7 +14,7 @@ from test_gpu_gateup import _check, _inputs, ppas  # noqa: F401
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("T", [1, 15, 16, 17, 33, 64, 65, 127, 128, 129])
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 33, 64, 65, 127, 128, 129, 145, 160, 161])
 @pytest.mark.parametrize("H,I", [(64, 128), (1024, 384)])
 def test_every_element_and_nothing_past_the_tokens(ppas, T, H, I):  # noqa: F811
     x, w = _inputs(T, H, I, seed=3 * T + H)
@@ -36,6 +36,7 @@ def test_every_element_and_nothing_past_the_tokens(ppas, T, H, I):  # noqa: F811
     (1, 64 * 25, 128),      # twice, and one
     (128, 64 * 6, 384),     # the long ring of 6 stages
     (128, 64 * 7, 384),
+    (160, 64 * 7, 128),
     (50, 64 * 20, 9728),    # a CTA for each of 152 SMs: the long ring
     (50, 64 * 20, 9856),    # two CTAs more: the short one
 ])
@@ -46,7 +47,7 @@ def test_ring_lengths(ppas, T, H, I):  # noqa: F811
 
 
 @pytest.mark.parametrize("T,H,I", [
-    (129, 64, 128 * 40),    # 40 tiles: one round of whole tiles
+    (161, 64, 128 * 40),    # 40 tiles: one round of whole tiles
     (200, 128, 128 * 30),   # 30 tiles: halves
     (256, 64, 128 * 19),    # 19 tiles: quarters
     (257, 192, 128),        # 2 tiles, the second of one token
