@@ -1007,8 +1007,8 @@ extern "C" ppas_status ppas_gateup_swiglu(const void *x, const void *w_packed, v
     gp.hidden = hidden;
     gp.inter = inter;
     gp.err = d_err_flag;
-    const bool few = n_tokens <= kFewTokens;
     const int sms = device_sm_count();
+    const bool few = n_tokens <= few_tokens(inter, sms);
     CUtensorMap tm_x, tm_w;
     if (!encode_bf16_2d(&tm_x, x, static_cast<uint64_t>(hidden), static_cast<uint64_t>(n_tokens), 64,
                         few ? static_cast<uint32_t>((n_tokens + 15) & ~15) : 128) ||

@@ -300,7 +300,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
 }
 
 // ---------------------------------------------------------------- few tokens
-// At most kFewTokens tokens (a decode iteration): the projection is bound by
+// At most few_tokens tokens (a decode iteration): the projection is bound by
 // streaming the weights, so the operands change sides.  A = weights, 64 gate
 // rows and the 64 up rows of the same features as one M128 tile; B = all the
 // tokens (N = tokens rounded up to 16).  One CTA per 64 features, two CTAs to
@@ -326,6 +326,9 @@ __host__ __device__ constexpr int few_stages(int n, uint32_t ring) {
 static_assert(few_stages(kFewTokens, kFewRing) >= 3, "ring depth");
 static_assert(kFewTokens * 128 * 4 <= few_stages(kFewTokens, kFewRing) * few_stage(kFewTokens),
               "epilogue buffer in the ring");
+static_assert(few_stages(kFewTokensAlone, kFewRingAlone) >= 3 && kFewTokensAlone <= 256 &&
+                  kFewTokensAlone * 128 * 4 <= few_stages(kFewTokensAlone, kFewRingAlone) * few_stage(kFewTokensAlone),
+              "the same where a CTA is alone");
 
 __global__ void __launch_bounds__(kGThreads, 2)
     gateup_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
@@ -497,7 +500,12 @@ cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, cons
 // 64 CTAs): 24 tokens 16.8 -> 14.1 us, 64: 20.6 -> 14.8, 128: 24.8 -> 17.9 (the
 // kernel above: 19.0, 19.2, 19.8); hidden 2048, inter 5632: 24 tokens 11.5 ->
 // 10.7, 128: 16.0 -> 12.7; hidden 1024, inter 2816: 128 tokens 6.7 -> 6.1, 24
-// tokens 4.9 and 4.9.
+// tokens 4.9 and 4.9.  This ring has five stages at 224 tokens; past 160, the
+// kernel above and this one: hidden 2048, inter 5632: 176 tokens 16.3 and 14.2,
+// 192: 16.3, 14.6, 224: 16.4, 15.6, 256: 16.7, 18.7; inter 9728: 192 tokens 19.9,
+// 18.2, 224: 20.0, 19.0; hidden 4096, inter 9728, 224 tokens: 31.8, 31.6.  With
+// fewer than half the SMs streaming it loses there: hidden 4096, inter 4096, 176
+// tokens: 20.1, 21.5.
 cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p, int sms,
                               cudaStream_t st) {
     static std::atomic<uint64_t> smem_set{0};

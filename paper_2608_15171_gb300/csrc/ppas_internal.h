@@ -290,8 +290,14 @@ bool encode_bf16_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t
 // tm_cut: of 128 / p.cut
 cudaError_t launch_gateup(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const CUtensorMap &tm_cut,
                           const GateUpParams &p, int pairs, cudaStream_t st);
-// calls of at most this many tokens take the weight-streaming kernel
-constexpr int kFewTokens = 160;
+// calls of at most this many tokens take the weight-streaming kernel: 64
+// features to a CTA, and more tokens where each CTA has an SM, and its longer
+// ring, to itself and half the SMs or more stream (both sides measured at
+// launch_gateup_few)
+constexpr int kFewTokens = 160, kFewTokensAlone = 224;
+inline int few_tokens(int inter, int sms) {
+    return inter / 64 <= sms && inter / 64 >= sms / 2 ? kFewTokensAlone : kFewTokens;
+}
 // tm_x: box of (n_tokens rounded up to 16) rows; tm_w: box of 64 rows
 cudaError_t launch_gateup_few(const CUtensorMap &tm_x, const CUtensorMap &tm_w, const GateUpParams &p, int sms,
                               cudaStream_t st);

@@ -1,5 +1,5 @@
 """The gate-up kernels at the edges of their ranges.  The weight-streaming one
-(calls of at most 160 tokens): one token, around each multiple of 16 that changes the
+(calls of at most 160 tokens, or 224): one token, around each multiple of 16 that changes the
 MMA's N, the largest call it takes and the first one past it; the smallest
 K and feature counts, and K longer than the ring.  Every element against the
 float64 oracle, and the rows after the last token untouched.  The CTA-pair
@@ -37,6 +37,10 @@ def test_every_element_and_nothing_past_the_tokens(ppas, T, H, I):  # noqa: F811
     (128, 64 * 6, 384),     # the long ring of 6 stages
     (128, 64 * 7, 384),
     (160, 64 * 7, 128),
+    (224, 64 * 6, 4864),    # half the SMs stream: the long ring of 5 stages up to 224 tokens
+    (193, 64 * 4, 9728),
+    (225, 64 * 6, 4864),    # and CTA pairs past that
+    (161, 64 * 6, 4736),    # fewer than half: CTA pairs past 160
     (50, 64 * 20, 9728),    # a CTA for each of 152 SMs: the long ring
     (50, 64 * 20, 9856),    # two CTAs more: the short one
 ])
@@ -47,7 +51,7 @@ def test_ring_lengths(ppas, T, H, I):  # noqa: F811
 
 
 @pytest.mark.parametrize("T,H,I", [
-    (161, 64, 128 * 40),    # 40 tiles: one round of whole tiles
+    (225, 64, 128 * 40),    # 40 tiles: one round of whole tiles
     (200, 128, 128 * 30),   # 30 tiles: halves
     (256, 64, 128 * 19),    # 19 tiles: quarters
     (257, 192, 128),        # 2 tiles, the second of one token
