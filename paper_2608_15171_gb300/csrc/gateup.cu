@@ -58,9 +58,10 @@ enum : int {
     G_COUNT = G_DRAIN + 1
 };
 constexpr uint32_t kOffTmemG = kOffBarG + G_COUNT * 8;
-constexpr uint32_t kOffAbortG = kOffTmemG + 4;
+constexpr uint32_t kOffAbortG = kOffTmemG + 4;   // set in both CTAs of a pair
+constexpr uint32_t kOffIssuedG = kOffAbortG + 4;  // K blocks whose copies this CTA issued
 constexpr uint32_t kSmemG = kOffBarG + 256 + 1024;  // + alignment slack
-static_assert(kOffAbortG + 4 <= kOffBarG + 256, "barrier area");
+static_assert(kOffIssuedG + 4 <= kOffBarG + 256, "barrier area");
 static_assert(kSmemG <= 232448, "shared memory per CTA");
 constexpr int kGThreads = 192;
 
@@ -140,6 +141,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
     const int k_blocks = p.hidden / kGK;
     const uint32_t rank = cluster_ctarank();  // 0: the pair's leader
     const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    // a wait ran out: both CTAs of the pair are told
+    auto give_up = [&]() {
+        *abort_flag = 1;
+        dsmem_st_s32(dsmem_addr(sb + kOffAbortG, rank ^ 1u), 1);
+    };
 
     if (warp == 1) {
         tmem_alloc_pair(sb + kOffTmemG, 512);
@@ -202,7 +208,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
         // the leader's last releases of the ring have reached this CTA before it leaves
         for (int j = max(0, q - kGStages); ok && j < q; ++j)
             ok = mbar_wait_warp(bar(G_EMPTY + j % kGStages), (j / kGStages) & 1, p.err);
-        if (!ok) *abort_flag = 1;
+        if (!ok) give_up();
+        if (lane == 0) *reinterpret_cast<volatile int *>(sg + kOffIssuedG) = q;
         // every MMA of the pair has completed, and this CTA has been told
         mbar_wait_warp(bar(G_DRAIN), 0, p.err);
     } else if (warp == 1) {
@@ -241,7 +248,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
                     __syncwarp();
                 }
             }
-            if (!ok) *abort_flag = 1;
+            if (!ok) give_up();
             if (elect_one()) umma_commit_pair(bar(G_DRAIN));
         }
     } else {
@@ -254,7 +261,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
             const bool ok = mbar_wait_warp(bar(G_ACCFULL + buf), (it >> 1) & 1, p.err) &&
                             !__any_sync(0xffffffffu, *abort_flag);
             if (!ok) {
-                *abort_flag = 1;
+                give_up();
                 break;
             }
             tc_fence_after();
@@ -293,6 +300,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
     tc_fence_before();
     __syncwarp();
     cluster_sync_all();
+    if (*abort_flag) {  // (the same in both CTAs)
+        // after a timeout, nor while copies are in flight: the leader, whose
+        // barriers count both CTAs' bytes, waits for the newest block of each
+        // stage, and arms what only the other CTA issued
+        if (rank == 0 && warp == 0) {
+            const int q0 = *reinterpret_cast<volatile int *>(sg + kOffIssuedG);
+            const int q1 = dsmem_ld_s32(dsmem_addr(sb + kOffIssuedG, 1));
+            const RingPairNewest nw =
+                lane < kGStages ? ring_pair_newest(q0, q1, lane, kGStages) : RingPairNewest{-1, false};
+            if (nw.arm) {
+                const GateUpItem item = gateup_item(p, pair + nw.block / k_blocks * n_pairs, m_blocks, n_blocks);
+                mbar_expect_tx(bar(G_FULL + lane), kABytes + static_cast<uint32_t>(item.width) * kGK * 2);
+            }
+            if (nw.block >= 0) mbar_wait(bar(G_FULL + lane), (nw.block / kGStages) & 1, nullptr);
+            __syncwarp();
+        }
+        cluster_sync_all();
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem, 512);
@@ -379,7 +404,8 @@ __global__ void __launch_bounds__(kGThreads, 2)
     grid_dep_launch();
 
     if (warp == 0) {
-        for (int kb = 0, s = 0, round = 0; kb < k_blocks; ++kb) {
+        int kb = 0;
+        for (int s = 0, round = 0; kb < k_blocks; ++kb) {
             if (round > 0 && !mbar_wait_warp(empty(s), (round - 1) & 1, p.err)) {
                 *abort_flag = 1;
                 break;
@@ -397,6 +423,7 @@ __global__ void __launch_bounds__(kGThreads, 2)
                 ++round;
             }
         }
+        ring_land(full(0), kb, stages, lane);
     } else if (warp == 1) {
         const uint64_t da0 = smem_desc_sw128(sb, 16, 1024);
         const uint64_t db0 = smem_desc_sw128(sb + kFewA, 16, 1024);

@@ -83,6 +83,17 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, in
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
 }
 
+// Waits, by a whole warp, until every copy that a producer issued into a ring
+// has landed (full0: the ring's first full barrier; lane s looks after stage s,
+// stages <= 32).  On every way out of a producer: nothing to wait for after an
+// ordinary end, since the consumer has waited for each block or is about to,
+// and after a timeout no copy of the CTA lands once it has left.
+__device__ __forceinline__ void ring_land(uint32_t full0, int issued, int stages, int lane) {
+    const int j = lane < stages ? ring_newest(issued, lane, stages) : -1;
+    if (j >= 0) mbar_wait(full0 + 8u * static_cast<uint32_t>(lane), (j / stages) & 1, nullptr);
+    __syncwarp();
+}
+
 // ---------------------------------------------------------------- named barriers
 // bar.sync / bar.arrive on a named barrier (0 is __syncthreads); n counts
 // threads (a multiple of 32) and every warp taking part executes it as a
@@ -127,6 +138,15 @@ __device__ __forceinline__ uint32_t dsmem_addr(uint32_t addr, uint32_t rank) {
 }
 __device__ __forceinline__ void dsmem_st_f32(uint32_t addr, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+__device__ __forceinline__ void dsmem_st_s32(uint32_t addr, int32_t v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ int32_t dsmem_ld_s32(uint32_t addr) {
+    int32_t v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
 }
 
 // arrive on an mbarrier of another CTA of the cluster (addr from dsmem_addr)

@@ -23,6 +23,33 @@ constexpr int kPageBytes = kPage * kRowBytes;  // one (block, kv-head) page: 4 K
 // device the plans are made for its SM count (plan_sms()).
 constexpr int32_t kDefaultPlanSms = 152;
 
+// ------------------------------------------------------------------ TMA rings
+// Block j of a ring goes through stage j % stages.  A kernel whose bounded wait
+// ran out leaves only when the copies it has issued have landed (each is
+// waited for, again within the limit): which block's phase that is, per stage.
+
+// The newest of `issued` blocks that went through stage s; -1 when none did.
+// No later block uses that stage's barrier, so a wait for its phase covers it
+// whether or not the block was consumed.
+__host__ __device__ constexpr int ring_newest(int issued, int s, int stages) {
+    return issued <= s ? -1 : s + (issued - 1 - s) / stages * stages;
+}
+
+// The same for a ring that two CTAs fill and the first one's barriers count
+// (that CTA arms a block's phase for both as it issues its own part): blocks
+// issued by the first and by the second CTA.  arm: only the second one issued
+// the block, so its part has to be armed before the wait.  (The second is never
+// a whole round ahead: it reuses a stage once the block before was consumed,
+// which takes both parts.)
+struct RingPairNewest {
+    int block;
+    bool arm;
+};
+__host__ __device__ constexpr RingPairNewest ring_pair_newest(int issued0, int issued1, int s, int stages) {
+    const int a = ring_newest(issued0, s, stages), b = ring_newest(issued1, s, stages);
+    return {a < b ? b : a, a < b};
+}
+
 // ------------------------------------------------------------------ prefill
 // Rows with q_len > 1.  The kernel is persistent: one CTA per SM works
 // through a list of items, each one 128-token query tile of heads_per_cta
