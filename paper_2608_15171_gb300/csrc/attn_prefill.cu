@@ -333,6 +333,9 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
     // the set-up above overlaps the previous kernel of the stream; global
     // memory (KV pages, Q, block tables, outputs) only after it has completed
     grid_dep_wait();
+    // KV tiles whose copies this producer has issued; the Q loader's Q tiles (tile n
+    // of them has the barrier B_Q + n % hpc)
+    int issued = 0;
 
     if (warp < 4) {
         // ------------------------------------------------------------ K/V producers
@@ -356,7 +359,8 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
             int w = w_beg, jj = 0;
             ItemView cur = item_view(p, w);
             load_id(cur, 0);
-            for (int g = 0;; ++g) {
+            for (;;) {
+                const int g = issued;
                 const int s = g % ns;
                 const int np = max(0, min(kPagesPerTile / 2, pages_in(cur.ctx_len, cur.kt0 + jj) - pg_lo));
                 if (pg - pg_lo < np && (id < 0 || id >= p.num_blocks)) {
@@ -392,6 +396,7 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                         }
                 }
                 __syncwarp();
+                ++issued;
                 if (!more) break;
                 w = wn;
                 jj = jn;
@@ -516,6 +521,7 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
                         tma_load_3d(sb + kOffQ + t * kTileBytes + kHalf, &tm_q, 64, h0 + t, qrow, bar(B_Q + t));
                     }
                     __syncwarp();
+                    ++issued;
                 }
                 if (!ok) {
                     *abort_flag = 1;
@@ -720,6 +726,13 @@ __device__ __forceinline__ void prefill_cta(const CUtensorMap &tm_q, const CUten
     if (warp == kMmaWarp) {
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
+    }
+    // a wait ran out: the copies in flight land before the CTA leaves.  (Last, and
+    // once for all rings: before the release of TMEM, or by each producer at its
+    // end, it cost a step of short items, or a long one, 0.3-1 %.)
+    if (*abort_flag && issued > 0) {
+        const bool q = warp == kQWarp, v = warp >= 2;
+        ring_land(bar(q ? B_Q : v ? B_VFULL : B_KFULL), issued, q ? hpc : v ? kNV : kNK, lane);
     }
 }
 

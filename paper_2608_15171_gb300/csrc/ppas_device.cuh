@@ -83,14 +83,30 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, in
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
 }
 
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Waits, by a whole warp, until every copy that a producer issued into a ring
 // has landed (full0: the ring's first full barrier; lane s looks after stage s,
-// stages <= 32).  On every way out of a producer: nothing to wait for after an
-// ordinary end, since the consumer has waited for each block or is about to,
-// and after a timeout no copy of the CTA lands once it has left.
+// stages <= 32), so that none lands once the CTA has left.  After an ordinary
+// end there is nothing to wait for: each block's consumer waited for it, or is
+// about to.  (A block that two warps fetch and only one got to is waited for
+// until the limit, 0.2 s or more.  No clock and no error word: little code.)
 __device__ __forceinline__ void ring_land(uint32_t full0, int issued, int stages, int lane) {
     const int j = lane < stages ? ring_newest(issued, lane, stages) : -1;
-    if (j >= 0) mbar_wait(full0 + 8u * static_cast<uint32_t>(lane), (j / stages) & 1, nullptr);
+    bool landed = j < 0;
+#pragma unroll 1
+    for (int i = 0; !landed && i < (1 << 24); ++i)
+        landed = mbar_test_wait(full0 + 8u * static_cast<uint32_t>(lane), (j / stages) & 1);
     __syncwarp();
 }
 

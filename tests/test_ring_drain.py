@@ -28,6 +28,7 @@ def test_waits_cover_every_copy_in_flight(tmp_path):
 @pytest.mark.parametrize("source,kernel,wait", [
     ("gateup.cu", "gateup_swiglu_kernel", "ring_pair_newest("),
     ("gateup.cu", "gateup_few_kernel", "ring_land("),
+    ("attn_prefill.cu", "prefill_cta", "ring_land(bar(q ? B_Q : v ? B_VFULL : B_KFULL)"),
 ])
 def test_kernels_wait_for_them(source, kernel, wait):
     with open(os.path.join(CSRC, source)) as f:
