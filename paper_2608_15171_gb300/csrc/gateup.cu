@@ -92,24 +92,6 @@ __device__ __forceinline__ void tmem_ld16_sync(uint32_t taddr, uint32_t (&r)[16]
         : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32_wait(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-          "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-          "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-          "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // item t of the launch: the first n_full are whole tiles, the others slices
 __device__ __forceinline__ GateUpItem gateup_item(const GateUpParams &p, int t, int m_blocks, int n_blocks) {
     GateUpItem it;
@@ -271,8 +253,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
 #pragma unroll 1
             for (int c = 0; c < item.width / 32; ++c) {
                 float gv[32], uv[32];
-                tmem_ld32_wait(t_lane + buf * kGN + c * 32, gv);
-                tmem_ld32_wait(t_lane + buf * kGN + item.width + c * 32, uv);
+                tmem_ld32_sync(t_lane + buf * kGN + c * 32, gv);
+                tmem_ld32_sync(t_lane + buf * kGN + item.width + c * 32, uv);
                 if (row0 + lane < p.n_tokens) {
                     uint4 *dst = reinterpret_cast<uint4 *>(out + static_cast<int64_t>(lane) * p.inter + c * 32);
 #pragma unroll
