@@ -522,7 +522,7 @@ PrefillPlan plan_prefill(int32_t n_seqs, const int32_t *q_lens, const int32_t *c
 }
 
 int32_t decode_reserve_sms(int32_t n_seqs, const int32_t *q_lens, const int32_t *ctx_lens, int32_t n_q_heads,
-                           int32_t n_kv_heads, int32_t num_sms) {
+                           int32_t n_kv_heads, int32_t num_sms, const DecodePlan *plain) {
     const int32_t hpc = n_q_heads / n_kv_heads >= 2 ? 2 : 1;
     const int64_t slots = n_q_heads / hpc;
     double units = 0.0, bytes = 0.0;  // prefill KV tiles x head slots, decode K/V bytes
@@ -550,9 +550,10 @@ int32_t decode_reserve_sms(int32_t n_seqs, const int32_t *q_lens, const int32_t 
     // SM would be its tail, so all of them get one at once.  (512 tokens over
     // 2048 with 2 decode rows, 32 splits: with 8 SMs left to them 8 of the 32
     // would start when the first ones end.)
-    const DecodePlan d = plan_decode(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, num_sms);
-    const double split_us = kDecodeSplitUs + bytes / static_cast<double>(d.n_ctas) / kDecodeBytesPerSmUs;
-    if (sm_time / num_sms < 2 * split_us) k = std::max(k, static_cast<int32_t>(std::min<int64_t>(d.n_ctas, num_sms)));
+    const int64_t splits =
+        plain ? plain->n_ctas : plan_decode(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, num_sms).n_ctas;
+    const double split_us = kDecodeSplitUs + bytes / static_cast<double>(splits) / kDecodeBytesPerSmUs;
+    if (sm_time / num_sms < 2 * split_us) k = std::max(k, static_cast<int32_t>(std::min<int64_t>(splits, num_sms)));
     return std::max(0, std::min(k, num_sms / 2));
 }
 
@@ -593,29 +594,23 @@ StepPlan plan_step(int32_t n_seqs, const int32_t *q_lens, const int32_t *ctx_len
                    int32_t n_kv_heads, size_t workspace_bytes) {
     StepPlan sp;
     const int32_t sms = plan_sms();
-    sp.n_ctas = sms - decode_reserve_sms(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, sms);
-    // true when the workspace holds everything the plan wants
-    auto plan_with = [&](bool fine_tail) {
-        sp.dp = plan_decode(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, sms, decode_cluster_caps(), fine_tail);
-        const bool may_mix = !sp.dp.rows.empty() && sp.dp.rows.size() <= static_cast<size_t>(kMaxMixedRows);
-        bool full = true;
-        auto plan = [&](int32_t max_work) {
-            PrefillPlan pf =
-                plan_prefill(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, true, sp.n_ctas, max_work);
-            // a workspace too small for the pieces' partials runs every unit whole
-            if (workspace_bytes < sp.dp.total_bytes() + pf.total_bytes()) {
-                full = false;
-                pf = plan_prefill(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, false, sp.n_ctas, max_work);
-            }
-            return pf;
-        };
-        sp.pf = plan(may_mix ? kMaxMixedWork : kMaxPrefillWork);
-        sp.mixed = may_mix && sp.pf.launches.size() == 1;
-        if (may_mix && !sp.mixed) sp.pf = plan(kMaxPrefillWork);  // several prefill launches anyway
-        return full;
-    };
-    // a workspace short of the finer splits' partials gets the coarser plan
-    if (!plan_with(true)) plan_with(false);
+    const DecodeClusterCaps caps = decode_cluster_caps();
+    sp.dp = plan_decode(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, sms, caps);
+    sp.n_ctas = sms - decode_reserve_sms(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, sms, &sp.dp);
+    // one prefill plan, whichever decode plan goes with it (planning is host
+    // time of every iteration, most of it this one's search)
+    static_assert(kMaxMixedWork == kMaxPrefillWork, "a mixed launch takes the items of a prefill launch");
+    sp.pf = plan_prefill(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, true, sp.n_ctas);
+    if (!sp.dp.rows.empty() && !sp.pf.empty()) {
+        // a workspace short of the finer splits' partials keeps the coarser plan
+        DecodePlan fine = plan_decode(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, sms, caps, true);
+        if (workspace_bytes >= fine.total_bytes() + sp.pf.total_bytes()) sp.dp = std::move(fine);
+    }
+    // a workspace too small for the pieces' partials runs every unit whole
+    if (workspace_bytes < sp.dp.total_bytes() + sp.pf.total_bytes())
+        sp.pf = plan_prefill(n_seqs, q_lens, ctx_lens, n_q_heads, n_kv_heads, false, sp.n_ctas);
+    sp.mixed = !sp.dp.rows.empty() && sp.dp.rows.size() <= static_cast<size_t>(kMaxMixedRows) &&
+               sp.pf.launches.size() == 1;
     return sp;
 }
 

@@ -161,9 +161,11 @@ struct PrefillPlan {
 
 // SMs the persistent prefill kernel leaves to the decode launch of the same
 // step on a device of num_sms SMs (0 without decode rows or without prefill
-// chunks)
+// chunks).  plain: the step's plan_decode() without finer splits, made here when
+// the caller has none.
+struct DecodePlan;
 int32_t decode_reserve_sms(int32_t n_seqs, const int32_t *q_lens, const int32_t *ctx_lens, int32_t n_q_heads,
-                           int32_t n_kv_heads, int32_t num_sms);
+                           int32_t n_kv_heads, int32_t num_sms, const DecodePlan *plain = nullptr);
 
 // n_ctas: CTAs (SMs) the persistent kernel may occupy; allow_split == false
 // keeps every unit whole (no workspace); max_work: items a launch may take
