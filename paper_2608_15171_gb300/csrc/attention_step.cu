@@ -224,24 +224,32 @@ DecodePlan plan_decode(int32_t n_seqs, const int32_t *q_lens, const int32_t *ctx
     // Beside prefill items the decode CTAs come one after another, in row
     // order, as SMs take them, and when the items are done those that are left
     // run at once, at an SM's rate each: the step ends a whole split later.
-    // So the splits of the last third of the rows are half as long.  Per step:
-    // 4 x 512 + 8 rows (16/2 heads) 131.9 -> 128.8 us, 3 x 683 + 16 rows (32/8)
-    // 610 -> 595, 1024 + 16 rows 100.0 -> 98.0 (16/2) and 290.5 -> 283.4 (32/8),
-    // 2 x 256 + 30 rows 119.8 -> 111.7, 512 + 16 rows 76.0 -> 74.0.  (The last half:
-    // 130.2, 596; all rows: 138, 630; thirds instead of halves: 130.7, 594.)
-    // Not for steps of many splits already, whose scratch would grow, nor for
-    // short splits, where a second one costs more than the tail (69 rows of ~90
-    // pages + 277 tokens, 8/8 heads: 66.0 -> 68.6 us).
+    // So the splits of the last third of the rows are half as long.  Per step,
+    // plain and halved: 4 x 512 + 8 rows (16/2 heads) 131.9 -> 128.8 us, 3 x 683 +
+    // 16 rows (32/8) 610 -> 595, 1024 + 16 rows 100.0 -> 98.0 (16/2) and 290.5 ->
+    // 283.4 (32/8), 2 x 256 + 30 rows 119.8 -> 111.7, 512 + 16 rows 76.0 -> 74.0.  (The
+    // last half: 130.2, 596; all rows: 138, 630; thirds instead of halves: 130.7,
+    // 594.)  Where the decode launch goes to a side stream the end is the same:
+    // 512 + 130 rows (16/2) 355.5 -> 344.5, 17,000 + 16 rows (32/8) 1498 -> 1487, 20,000
+    // + 8 rows 1993 -> 1992.
+    // At most four splits an SM in all, the last rows first: the end is then
+    // short by itself, and a second split of a few thousand tokens costs more
+    // (512 + 70 rows of 3200 tokens, 32/8: 560 plain splits 140.3 us, all 744 of
+    // them 141.6, up to the limit 140.4; 700 + 76 rows 144.6, 146.6, 144.6).  Nor for
+    // short splits (69 rows of ~90 pages + 277 tokens, 8/8 heads: 66.0 -> 68.6 us).
     if (fine_tail && static_cast<int32_t>(nr) != n_seqs) {
         int64_t ctas = 0;
         for (size_t k = 0; k < nr; ++k) ctas += static_cast<int64_t>(ns1[k]) * n_kv_heads;
-        for (size_t k = nr - nr / 3; k < nr && ctas <= 4 * static_cast<int64_t>(num_sms); ++k) {
+        for (size_t k = nr; k-- > nr - nr / 3;) {
             const int64_t pages = (ctx_lens[d.rows[k]] + kPage - 1) / kPage;
             if (pps1[k] < kDecodeMinPagesToHalve) continue;
             const int64_t want = 2 * static_cast<int64_t>(ns1[k]);
             const int64_t pps = std::max<int64_t>(kDecodeMinPagesPerSplit, (pages + want - 1) / want);
+            const int64_t ns = (pages + pps - 1) / pps;
+            ctas += (ns - ns1[k]) * n_kv_heads;
+            if (ctas > 4 * static_cast<int64_t>(num_sms)) break;
             pps1[k] = static_cast<int32_t>(pps);
-            ns1[k] = static_cast<int32_t>((pages + pps - 1) / pps);
+            ns1[k] = static_cast<int32_t>(ns);
         }
     }
     d.n_splits = ns1;
