@@ -282,10 +282,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
     tc_fence_before();
     __syncwarp();
     cluster_sync_all();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem, 512);
+    }
     if (*abort_flag) {  // (the same in both CTAs)
-        // after a timeout, nor while copies are in flight: the leader, whose
+        // a wait ran out: nor while copies are in flight.  The leader, whose
         // barriers count both CTAs' bytes, waits for the newest block of each
-        // stage, and arms what only the other CTA issued
+        // stage, and arms what only the other CTA issued.  (After the release of
+        // TMEM: before it, calls of 10 us took 0.05 more.)
         if (rank == 0 && warp == 0) {
             const int q0 = *reinterpret_cast<volatile int *>(sg + kOffIssuedG);
             const int q1 = dsmem_ld_s32(dsmem_addr(sb + kOffIssuedG, 1));
@@ -299,10 +304,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
             __syncwarp();
         }
         cluster_sync_all();
-    }
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc_pair(tmem, 512);
     }
 }
 
