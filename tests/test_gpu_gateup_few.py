@@ -76,6 +76,54 @@ def test_pair_tiles_and_slices_of_the_last_round(ppas, T, H, I):  # noqa: F811
            f"T={T} H={H} I={I}")
 
 
+@pytest.mark.parametrize("T,H,I", [
+    (160, 64 * 7, 11008),   # two CTAs on most SMs: all 512 TMEM columns, three stages, the epilogue over them
+    (129, 64 * 4, 11008),
+    (144, 64 * 3, 9856),    # just more CTAs than SMs, K as long as the ring
+    (8, 2048, 11008),       # a decode iteration
+    (64, 64 * 8, 20480),    # 320 CTAs: more than two for each SM
+])
+def test_shared_sms_back_to_back(ppas, T, H, I):  # noqa: F811
+    """More CTAs than SMs, each call started while the one before still runs."""
+    x, w = _inputs(T, H, I, seed=T + H + I)
+    wp = torch.empty_like(w)
+    ppas.ppas_gateup_pack(w, wp, H, I)
+    ys = [torch.full((T + 3, I), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(6)]
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for y in ys:
+        ppas.ppas_gateup_swiglu(x, wp, y, T, H, I, err)
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    for y in ys:
+        assert bool((y[T:] == 7.0).all()) and torch.equal(y, ys[0])
+    _check(ys[0][:T].float().cpu().numpy(), mlp.gate_up(x.float().cpu().numpy(), w.float().cpu().numpy()),
+           f"T={T} H={H} I={I}")
+
+
+def test_both_kernels_in_turn_on_one_stream(ppas):  # noqa: F811
+    """Calls of 8, 160 and 300 tokens (rings of other depths, one and two CTAs
+    an SM, CTA pairs) after one another without a wait equal the same calls
+    with one."""
+    H, I = 64 * 10, 11008
+    x, w = _inputs(300, H, I, seed=5)
+    wp = torch.empty_like(w)
+    ppas.ppas_gateup_pack(w, wp, H, I)
+    got = []
+    for wait in (True, False):
+        ys = []
+        torch.cuda.synchronize()
+        for T in (8, 160, 300) * 4:
+            y = torch.full((T, I), 7.0, dtype=torch.bfloat16, device="cuda")
+            ppas.ppas_gateup_swiglu(x[:T], wp, y, T, H, I)
+            if wait:
+                torch.cuda.synchronize()
+            ys.append(y)
+        torch.cuda.synchronize()
+        got.append(ys)
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+    _check(got[0][2].float().cpu().numpy(), mlp.gate_up(x.float().cpu().numpy(), w.float().cpu().numpy()), "300 tokens")
+
+
 def test_back_to_back_calls_on_each_others_output(ppas):  # noqa: F811
     """Each call reads what the call before wrote (the kernel sets up while
     its predecessor still runs): a chain of calls equals the same chain with
