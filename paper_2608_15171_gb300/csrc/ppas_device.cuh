@@ -165,9 +165,12 @@ __device__ __forceinline__ int32_t dsmem_ld_s32(uint32_t addr) {
     return v;
 }
 
-// arrive on an mbarrier of another CTA of the cluster (addr from dsmem_addr)
+// Arrive on an mbarrier of another CTA of the cluster (addr from dsmem_addr),
+// without a cluster-scope release: that waits until the thread's earlier global
+// stores have been performed, about 1 us behind an epilogue's.  For arrivals
+// that hand over no memory of either CTA.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
 // ---------------------------------------------------------------- TMA

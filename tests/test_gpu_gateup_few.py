@@ -76,6 +76,25 @@ def test_pair_tiles_and_slices_of_the_last_round(ppas, T, H, I):  # noqa: F811
            f"T={T} H={H} I={I}")
 
 
+@pytest.mark.parametrize("T,H,I", [(4000, 64, 128 * 54), (2500, 512, 128 * 31)])
+def test_many_rounds_of_short_tiles(ppas, T, H, I):  # noqa: F811
+    """Many rounds of the CTA-pair kernel with little K: the epilogue sets the
+    pace, and the next tile's MMAs wait for it to leave each accumulator."""
+    x, w = _inputs(T, H, I, seed=T + H)
+    wp = torch.empty_like(w)
+    ppas.ppas_gateup_pack(w, wp, H, I)
+    ys = [torch.full((T + 1, I), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(4)]
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for y in ys:
+        ppas.ppas_gateup_swiglu(x, wp, y, T, H, I, err)
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    for y in ys:
+        assert bool((y[T:] == 7.0).all()) and torch.equal(y, ys[0])
+    _check(ys[0][:T].float().cpu().numpy(), mlp.gate_up(x.float().cpu().numpy(), w.float().cpu().numpy()),
+           f"T={T} H={H} I={I}")
+
+
 @pytest.mark.parametrize("T,H,I", [
     (160, 64 * 7, 11008),   # two CTAs on most SMs: all 512 TMEM columns, three stages, the epilogue over them
     (129, 64 * 4, 11008),
