@@ -499,11 +499,12 @@ PrefillPlan plan_prefill(int32_t n_seqs, const int32_t *q_lens, const int32_t *c
                     per_cta[c].push_back(pc.second);
                 }
             const int64_t cut_span = span(filled);
-            // the partials and the merge cost kPrefillMergeCost tiles, two more in
-            // a step of 64 tiles a CTA or longer, where many CTAs write them at
-            // once (2048 tokens, longest CTA 19 tiles against 14 cut: 26.1 us a
+            // the partials and the merge cost kPrefillMergeCost tiles, one more
+            // where the longest CTA of whole units has 32 tiles, two from 64 on:
+            // more CTAs then write partials at the same time.  (Fitted to two
+            // steps: 2048 tokens, longest CTA 19 tiles against 14 cut: 26.1 us a
             // layer whole, 25.0 cut; 16384 tokens, 464 against about 458: 640 whole,
-            // 655 cut)
+            // 655 cut.)
             const int64_t cost = kPrefillMergeCost + std::min<int64_t>(2, whole_span / 32);
             if (lp.n_part == 0 || (!needs_cut && cut_span + cost >= whole_span)) {
                 per_cta = std::move(whole);  // not worth the partials
@@ -571,7 +572,7 @@ int32_t decode_reserve_sms(int32_t n_seqs, const int32_t *q_lens, const int32_t 
 // inter 11008) over 76 pairs 28.7 -> 25.0 us, 774 (2056 tokens) 113.1 -> 108.8.
 // A slice takes more than its share (every slice reads the tile's tokens), so
 // slices over several rounds lose: 344 tiles (800 tokens), the last 40 as 160
-// quarters, 57.5 us against 54.5 whole.
+// quarters, 57.5 us against 54.5 whole.  (Runs of a few ms.)
 GateUpPlan plan_gateup(int32_t n_tokens, int32_t inter, int32_t max_pairs) {
     const int64_t tiles = (static_cast<int64_t>(n_tokens) + 255) / 256 * (inter / 128);
     const int64_t last = tiles % max_pairs;  // tiles of the last round

@@ -35,7 +35,7 @@
 // loads, and the last CTA merges up to 20 partials in one round, weights in
 // registers.  One row x 25k, 16/2 heads, append + attention: 14.3 -> 12.8 us
 // a layer; 8 rows x 25k 37.4 -> 36.8.  (Claiming at entry cost
-// the page loop 1 %: 96 rows of 17-4100 tokens 270.8 -> 274.5 us.)
+// the page loop 1 %: 96 rows of 17-4100 tokens 135.4 -> 137.3 us a layer.)
 #include <math.h>
 
 #include "ppas_device.cuh"
@@ -493,7 +493,10 @@ __device__ __forceinline__ void decode_cta(const CUtensorMap &tm_k, const CUtens
         for (int o_ = 16; o_ >= 1; o_ >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o_);
         return x;
     };
-    constexpr int kBatch = 20;  // a one-row step in clusters has 18 or 19 partials: one round
+    // partials a round: as many as the registers hold beside the rest (4 each).
+    // A one-row step in clusters of 4 has 18 with 2 kv-heads (one round), 36 with
+    // 1 (two, by the other path), fewer with more.
+    constexpr int kBatch = 20;
     float4 ov[kBatch];
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float L;

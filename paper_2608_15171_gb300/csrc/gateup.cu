@@ -11,10 +11,16 @@
 // the SM and the [T, 2I] intermediate never reaches HBM.  Each CTA of the pair
 // loads its own tokens and half of the weight rows: 32 KB of L2 traffic for 64
 // columns of K and 512 tensor cycles.  A CTA by itself with the same 128 x 256
-// share needs 48 KB, 96 B/clk on every SM, which L2 does not deliver (2056
-// tokens, hidden 2048, inter 11008: 118.1 us; the pairs take 108.8, 16,384
-// tokens 815 -> 740 us in a short run, 896 -> 838 at the power limit of a long
-// one; 1024 tokens 66.0 -> 55.8, 256 33.2 -> 25.0).
+// share needs 48 KB, 96 B/clk on every SM, which L2 does not deliver.  Hidden
+// 2048, inter 11008, 128-token tiles of single CTAs and now, us; a run of a few
+// ms, and back to back for 150 ms (the GPU is then at its power limit):
+//   256 tokens  34.0 -> 24.7, 33.8 -> 24.7     2056  119.3 -> 105.8, 128.8 -> 122.0
+//   512         43.3 -> 32.0, 43.1 -> 35.3    16384  818 -> 721, 908 -> 854
+//   1024        66.5 -> 54.5, 68.2 -> 62.4
+// Tokens are padded to 256 instead of 128, so that calls of few rounds whose
+// last 128 tokens are all padding can be slower than those tiles were: 520
+// tokens 43.3 -> 44.1, 770 56.4 -> 58.7 (hidden 4096, inter 14336: 520 tokens 105.0
+// -> 108.5); most counts are faster (260 31.7 -> 30.2, 1030 76.6 -> 72.0).
 //
 // Persistent kernel, one CTA per SM, 192 threads:
 //   warp 0      TMA producer: X tile (128 x 64) and W tile (128 x 64) per
@@ -31,7 +37,7 @@
 // Tiles are visited in groups of 16 M blocks with the M block fastest, so
 // the pairs running at one time share a few weight tiles and keep a few MB of
 // X tiles hot in L2 (groups of 8: 2056 tokens 114.5 against 112.9 us).
-// Calls of at most kFewTokens tokens take another kernel, below.
+// Calls of at most few_tokens() tokens take another kernel, below.
 #include <algorithm>
 
 #include "ppas_device.cuh"
@@ -316,16 +322,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGThreads, 1)
 // At most few_tokens tokens (a decode iteration): the projection is bound by
 // streaming the weights, so the operands change sides.  A = weights, 64 gate
 // rows and the 64 up rows of the same features as one M128 tile; B = all the
-// tokens (N = tokens rounded up to 16).  One CTA per 64 features, two CTAs to
-// an SM, so that at inter = 11008 all 172 CTAs stream at once (tiles of 128
-// tokens x 128 features are 86, and pad the tokens to 128 rows of MMA work).
+// tokens (N = tokens rounded up to 16).  One CTA per 64 features.  Where those
+// are more than the SMs, two share one, so that at inter = 11008 all 172 CTAs
+// stream at once (tiles of 128 tokens x 128 features are 86, and pad the tokens
+// to 128 rows of MMA work); else each has an SM, and its memory, to itself.
 // 192 threads: warp 0 TMA, warp 1 MMA, warps 2-5 epilogue: gate and up
 // accumulators of a feature lie 64 TMEM lanes apart, so both go through shared
 // memory (the ring, once the last MMA has completed).
 // Hidden 2048, inter 11008 (90 MB of weights): see launch_gateup_few.
 constexpr int kFF = 64;  // features per CTA
 constexpr uint32_t kFewA = 128 * kGK * 2;  // weight tile of a K block: 16 KB
-constexpr uint32_t kFewRing = 112640;      // ring bytes at most: two CTAs share an SM
+constexpr uint32_t kFewRing = 112640;      // ring bytes at most where two CTAs share an SM
 constexpr uint32_t kFewRingAlone = 225280; // and where no SM gets a second CTA
 constexpr int kFewMaxStages = 12;
 

@@ -70,7 +70,7 @@ constexpr int kPrefillMinPiece = 4;     // shortest piece of a split unit, in KV
 // TMEM loses ~7e-7 of |O| per tile, so pieces are capped and the merge
 // (ordinary fp32) combines them
 constexpr int kPrefillMaxPiece = 512;
-constexpr int kPrefillMergeCost = 4;    // partial writes and the merge launch, in KV tiles
+constexpr int kPrefillMergeCost = 4;    // partial writes and the merge launch, in KV tiles (more in long steps)
 constexpr uint16_t kNoPart = 0xFFFF;    // an item of an unsplit unit
 
 struct PrefillSeq {
@@ -114,7 +114,8 @@ using PrefillParams = PrefillParamsT<kMaxPrefillWork>;
 static_assert(sizeof(PrefillParams) + 3 * 128 <= 32764, "kernel parameter space");
 
 // Merge of the split units' partials, launched after the prefill (or mixed)
-// launch: one thread per (split unit, head of the slot, query row, 4 columns).
+// launch: one thread per (split unit, head of the slot, query row, 8 columns),
+// the lanes of a warp on 32 rows.
 constexpr int kMaxMergeUnits = 1024;  // split units per merge launch
 
 struct MergeUnit {

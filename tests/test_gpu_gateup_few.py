@@ -1,9 +1,11 @@
 """The gate-up kernels at the edges of their ranges.  The weight-streaming one
-(calls of at most 160 tokens, or 224): one token, around each multiple of 16 that changes the
-MMA's N, the largest call it takes and the first one past it; the smallest
-K and feature counts, and K longer than the ring.  Every element against the
-float64 oracle, and the rows after the last token untouched.  The CTA-pair
-one: see there."""
+(calls of at most 160 tokens, 224 where each CTA has an SM and half the SMs or
+more have one): one token, around the multiples of 16 that change the MMA's N,
+the largest call it takes and the first one past it; the smallest K and
+feature counts, K around the length of each ring, and CTAs that share SMs,
+called back to back.  The CTA-pair one: last rounds whole and in slices, many
+rounds of little K.  Every element against the float64 oracle, and the rows
+after the last token untouched."""
 import numpy as np
 import pytest
 import torch
